@@ -322,7 +322,9 @@ KRON_API kron_status kron_autotune(kron_stream_t stream, int kind, int n, int64_
  * storage; scalar: every real storage type; the split tensor bodies below)
  * and KRON_ERR_INVALID_VALUE for
  * values out of range; all-zero restores the built-in default.  Strided,
- * transposed or misaligned batches always run the scalar body.  The 2-D split
+ * transposed, rectangular or misaligned batches (FP32 or 16-bit storage), and odd n
+ * with 16-bit storage, run the general-layout body, or the scalar body where that is
+ * set or measured faster.  The 2-D split
  * tensor path (KRON_COMPUTE_32F_BF16X3, FP32 or 16-bit storage) has two bodies:
  * KRON_VARIANT_IN_PLACE, one zero-padded 16 x 16 tile per instance (n <= 8:
  * several instances on the tile's diagonal), the second product taking the

@@ -255,6 +255,17 @@ static kron_status dispatch(KronDesc& d, cudaStream_t st) {
         const kron_status r = launch_fiberip(d, st);   // odd n, all contractions in place
         if (r != KRON_ERR_NOT_SUPPORTED) return r;
     }
+    // General layouts, and odd n with 16-bit storage.
+    if (d.variant != KRON_VARIANT_SCALAR && (!d.ycontig || ((d.N & 1) && d.io != KRON_R32F && d.beta == 0.0))) {
+        kron_status r = KRON_ERR_NOT_SUPPORTED;
+        switch (d.io) {
+            case KRON_R32F: r = d.D == 2 ? launch_span_f32_d2(d, st) : launch_span_f32_d3(d, st); break;
+            case KRON_R16BF: r = d.D == 2 ? launch_span_bf16_d2(d, st) : launch_span_bf16_d3(d, st); break;
+            case KRON_R16F: r = d.D == 2 ? launch_span_f16_d2(d, st) : launch_span_f16_d3(d, st); break;
+            default: break;
+        }
+        if (r != KRON_ERR_NOT_SUPPORTED) return r;
+    }
     switch (d.io) {
         case KRON_R32F: return d.D == 2 ? launch_fiber_f32_d2(d, st) : launch_fiber_f32_d3(d, st);
         case KRON_R64F: return d.D == 2 ? launch_fiber_f64_d2(d, st) : launch_fiber_f64_d3(d, st);

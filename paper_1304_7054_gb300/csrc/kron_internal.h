@@ -85,6 +85,15 @@ kron_status launch_fiber_c32_d3(const KronDesc& d, cudaStream_t s);
 kron_status launch_fiber_c64_d2(const KronDesc& d, cudaStream_t s);
 kron_status launch_fiber_c64_d3(const KronDesc& d, cudaStream_t s);
 
+// General layouts (padded, transposed, rectangular, any alignment) and odd n of the
+// 16-bit types; KRON_ERR_NOT_SUPPORTED where operands are mostly gaps.
+kron_status launch_span_f32_d2(const KronDesc& d, cudaStream_t s);
+kron_status launch_span_f32_d3(const KronDesc& d, cudaStream_t s);
+kron_status launch_span_bf16_d2(const KronDesc& d, cudaStream_t s);
+kron_status launch_span_bf16_d3(const KronDesc& d, cudaStream_t s);
+kron_status launch_span_f16_d2(const KronDesc& d, cudaStream_t s);
+kron_status launch_span_f16_d3(const KronDesc& d, cudaStream_t s);
+
 // Packed-pair FP32 kernels (even N, contiguous X and Y); KRON_ERR_NOT_SUPPORTED
 // for shapes they do not handle.
 kron_status launch_pair_f32_d2(const KronDesc& d, cudaStream_t s);
