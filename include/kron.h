@@ -88,7 +88,8 @@ typedef enum {
     KRON_COMPUTE_NATIVE = 0,
     /* Tensor cores, split precision: each FP32 value v = hi + lo with hi, lo
        bfloat16 (round to nearest even); products hi*hi + hi*lo + lo*hi are
-       accumulated in FP32.  Valid for R32F and R16BF storage. */
+       accumulated in FP32.  Valid for R32F and 16-bit storage.  Small n, where padding
+       to tensor tiles costs more than it saves, runs on the CUDA cores in FP32. */
     KRON_COMPUTE_32F_BF16X3 = 1
 } kron_compute;
 

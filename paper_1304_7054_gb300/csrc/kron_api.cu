@@ -212,8 +212,31 @@ static void choose_yvec(KronDesc& d) {
     }
 }
 
+// Split-precision calls that the CUDA-core bodies serve faster, in full FP32: the padding
+// of small instances to 16 x 16 tiles costs the tensor path more than the FMAs do here.
+// Measured (120 M elements, split -> FP32 bodies): FP32 storage 2-D n = 8: 255 -> 168 us,
+// n = 9: 381 -> 148, n = 14: 170 -> 156, n = 16: 148 -> 147 (stays); 3-D n = 4: 1878 -> 183,
+// n = 13: 343 -> 221, n = 14: 231 -> 229, n = 15: 223 -> 254 (stays).  16-bit storage 2-D n = 8:
+// 205 -> 143, n = 9: 293 -> 165, n = 10: 127 -> 154 (stays), n = 11: 217 -> 165, n = 13: 162 -> 188
+// (stays); 3-D n = 4: 1683 -> 153, n = 11: 330 -> 246, n = 12: 254 -> 231, n = 13: 256 -> 290 (stays).
+// Only calls that the split path itself takes are served (contiguous operands); with beta != 0
+// the FP32 bodies of 16-bit odd n are slower (old values of Y element by element), so the line
+// lies lower there.
+static bool cuda_cores_beat_split(const KronDesc& d) {
+    if (!d.contiguous || !d.ycontig) return false;
+    if (d.io != KRON_R32F && d.beta != 0.0 && (d.N & 1)) return d.N <= 7;
+    if (d.io == KRON_R32F) return d.D == 2 ? d.N <= 15 : d.N <= 14;
+    return d.D == 2 ? d.N <= 9 || d.N == 11 : d.N <= 12;
+}
+
 static kron_status dispatch(KronDesc& d, cudaStream_t st) {
     apply_tile_config(d);
+    // (a tile, depth or body set for the split path keeps it)
+    if (d.comp == KRON_COMPUTE_32F_BF16X3 && d.variant == KRON_VARIANT_AUTO && d.P <= 0 && d.nstage < 0 &&
+        d.warps <= 0 && d.fps <= 0 && cuda_cores_beat_split(d)) {
+        d.comp = KRON_COMPUTE_NATIVE;
+        apply_tile_config(d);
+    }
     if (d.io == KRON_C32F) return d.D == 2 ? launch_fiber_c32_d2(d, st) : launch_fiber_c32_d3(d, st);
     if (d.io == KRON_C64F) return d.D == 2 ? launch_fiber_c64_d2(d, st) : launch_fiber_c64_d3(d, st);
     if (d.comp == KRON_COMPUTE_32F_BF16X3) return launch_tc(d, st);
