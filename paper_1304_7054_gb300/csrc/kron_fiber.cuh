@@ -25,6 +25,7 @@
 // (Sec. 5 attributes the 3-D slowdown to it); here it never leaves the SM.
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
 
 #include "kron_complex.cuh"
@@ -418,6 +419,36 @@ size_t fiber_smem_bytes(int P, int nstage) {
            (size_t)P * (L::EX1 + L::EX2) * sizeof(T);
 }
 
+// Double precision runs at the rate of the DFMA units, one set per SM partition; warp w
+// of a CTA sits in partition w mod 4, so a stage takes as long as its fullest partition:
+// ceil(fibers / 128) rounds of 32-fiber warps (3-D n = 10: 3 instances fill 300 of 384
+// places, 5 fill 500 of 512).  Starting from about one fiber per thread (P0), the tiles
+// that just fill 1 to 10 rounds and fit in shared memory are taken when they save 5% of
+// the busiest SM's rounds, a tenth of a round counted for each tile's barriers and
+// copies (margins fitted on a sweep of all n: no n slower than P0, on average 2% off the
+// best tile).  Measured: 3-D n = 10, 65,536 instances 4750 -> 3984 us (0.78 -> 0.93 of
+// the 1.06 TFLOP/s DFMA peak), 2-D n = 12 (16 M elements) 1096 -> 784 us.
+template <typename T, typename S, int N, int D>
+int fiber_balanced_tile(int P0, int64_t batch, int sms, int nstage, size_t smem_limit) {
+    using L = FiberLayout<N, D>;
+    auto cost = [&](int P) {
+        const int64_t tiles = (batch + P - 1) / P, per_sm = (tiles + sms - 1) / sms;
+        return (double)per_sm * ((P * L::FPI + 127) / 128 + 0.1);
+    };
+    int best = P0;
+    double best_cost = cost(P0);
+    for (int r = 1; r <= 10; ++r) {
+        const int P = std::max(1, 128 * r / L::FPI);
+        if (P > 1 && fiber_smem_bytes<T, S, N, D>(P, nstage) > smem_limit) break;
+        const double c = cost(P);
+        if (c < 0.95 * best_cost) {
+            best = P;
+            best_cost = c;
+        }
+    }
+    return best;
+}
+
 template <typename T, typename S, int N, int D>
 kron_status launch_fiber_n(const KronDesc& d, cudaStream_t st) {
     using L = FiberLayout<N, D>;
@@ -462,13 +493,15 @@ kron_status launch_fiber_n(const KronDesc& d, cudaStream_t st) {
     // Instances per tile: about one fiber per thread and stage (tiles of any size
     // can be bulk-copied, see tile_span).  If the tile does not fit in shared
     // memory with a bulk-copy buffer, it is loaded element by element instead.
-    const int P0 = d.P > 0 ? d.P : (kFiberThreads + L::FPI - 1) / L::FPI;
-    int P = P0;
     int nstage = 0;
     if (d.contiguous) {
         nstage = d.nstage >= 1 ? d.nstage : 1;   // more resident CTAs beat a deeper pipeline (measured)
         if (nstage > 8) nstage = 8;
     }
+    constexpr bool dfma = std::is_same<T, double>::value || std::is_same<T, cf64>::value;
+    int P0 = d.P > 0 ? d.P : (kFiberThreads + L::FPI - 1) / L::FPI;
+    if (dfma && d.P <= 0) P0 = fiber_balanced_tile<T, S, N, D>(P0, d.batch, dev.sms, nstage, dev.smem_per_block_optin);
+    int P = P0;
     size_t smem = fiber_smem_bytes<T, S, N, D>(P, nstage);
     while (nstage > 1 && smem > dev.smem_per_block_optin) {
         --nstage;
