@@ -17,14 +17,14 @@
 // tile is contracted, the next one arrives in the other operand buffer by bulk
 // copies, one per instance: an instance starts anywhere (4-byte alignment for
 // FP32), so each copy takes the 16-byte-aligned span around it and the instance
-// sits at its alignment phase inside a 16-byte-aligned slot.  In 3-D the second
-// contraction writes over the dead operands and the last one into the exchange
-// buffer; in 2-D the last one writes over the dead operands.  Either way each
-// instance's results are contiguous, at the phase of its place in Y: the
-// 16-byte-aligned middle leaves by one bulk copy and the at most three elements
-// on either side by plain stores.  Global memory is thus read and written in
-// whole aligned granules, with no per-element address work.  Before the next
-// tile writes a buffer that outgoing copies still read, warp 0 waits for them.
+// sits at its alignment phase inside a 16-byte-aligned slot.  The first contraction
+// writes the exchange buffer, the second (3-D) rewrites its fibers in place there, and
+// the last one writes over the dead operands: each instance's results are contiguous,
+// at the phase of its place in Y: the 16-byte-aligned middle leaves by one bulk copy
+// and the at most three elements on either side by plain stores.  Global memory is
+// thus read and written in whole aligned granules, with no per-element address work.
+// The copies out of a buffer have a whole contraction of the next tile to finish
+// before warp 0 waits for them and refills the buffer; nobody else waits for them.
 //
 // Workspace (caller-owned device memory, written on the first execute with a
 // given pointer): tile table (int4: class key, first sorted index, count, 0),
@@ -45,7 +45,11 @@
 namespace kron {
 
 constexpr int kVlThreads = 256;
-constexpr int kVlBufBytes = 22528;                     // default budget of one buffer
+constexpr int kVlMaxP = 96;                            // instances per tile
+// Default budgets of one operand buffer and of the exchange buffer: four CTAs per SM
+// with one 3-D instance of n = 16, or two of n = 13.
+constexpr int kVlXBytes = 17664;
+constexpr int kVlEBytes = 18944;
 constexpr int kVlMaxBufBytes = 49152;                  // largest buffer a tuned tile may take
 constexpr int kVlKeys = 32;                            // class key = 16 (kind - 2) + n - 1
 
@@ -95,21 +99,16 @@ __device__ __forceinline__ int vl_nx(int key) {
 // Slot of one instance in an operand buffer: its elements plus up to 15 bytes
 // of alignment phase, rounded to 16 bytes.
 __host__ __device__ constexpr int vl_slot_bytes(int nx, int es) { return (nx * es + 15 + 15) / 16 * 16; }
-__host__ __device__ constexpr int vl_max(int a, int b) { return a > b ? a : b; }
-// Exchange elements of one instance (FP32): KP x N (2-D) or KP x N x N (3-D).
-__host__ __device__ constexpr int vl_exq(int kind, int n) { return vl_kp(n) * (kind == 2 ? n : n * n); }
-// Per-instance stride of the operand buffers (bytes).  In 3-D the second
-// contraction writes its FP32 exchange layout over the dead operands, so the
-// slot holds either.
+// Stride of mode 2 in the 3-D exchange buffer: 2 mod 4 words, so that lanes walking j
+// land on distinct even banks.
+__host__ __device__ constexpr int vl_js(int n) { return vl_kp(n) * n + (vl_kp(n) * n % 4 == 2 ? 0 : 2); }
+// Per-instance stride of the operand buffers (bytes): the operands, then the results.
 __host__ __device__ constexpr int vl_xs_bytes(int kind, int n, int es) {
-    return kind == 2 ? vl_slot_bytes(n * n, es)
-                     : (vl_max(vl_slot_bytes(n * n * n, es), 4 * vl_exq(3, n)) + 15) / 16 * 16;
+    return vl_slot_bytes(kind == 2 ? n * n : n * n * n, es);
 }
-// Per-instance stride of the exchange buffer (floats).  In 3-D the last
-// contraction writes the results there (contiguous, at their phase in Y), so a
-// slot is 16-byte aligned and holds either.
-__host__ __device__ constexpr int vl_e1_floats(int kind, int n, int es) {
-    return kind == 2 ? vl_exq(2, n) : (vl_max(vl_exq(3, n), vl_slot_bytes(n * n * n, es) / 4) + 3) / 4 * 4;
+// Per-instance stride of the exchange buffer (floats).
+__host__ __device__ constexpr int vl_e1_floats(int kind, int n) {
+    return kind == 2 ? vl_kp(n) * n : vl_js(n) * n;
 }
 
 // Alignment phase (in elements) of element offset `off` of an array at `base`.
@@ -225,18 +224,21 @@ __device__ __forceinline__ void vl_stage_out(S* dst, const f2 (&y)[vl_rows(N) / 
 
 // One tile of class (D, N) in operand buffer xt: instance q's operands at slot q,
 // phase vl_phase(X, xo[q]).  Its results, contiguous and column-major at phase
-// vl_phase(Y, yo[q]), go to operand slot q (2-D) or exchange slot q (3-D).
-// Exchange layouts put each stage's output pairs next to each other:
-//   2-D   W(l, j)    at j + KP l            in ex1  (stage 1 writes pairs along j)
-//   3-D   T(i, j, k) at k + KP i + KP N j   in ex1  (stage A: pairs along k)
-//         U(i, j, k) at j + KP k + KP N i   in xt   (stage B: pairs along j)
+// vl_phase(Y, yo[q]), go to the same slot, whose operands are dead by then.
+// Exchange layouts put the first stage's output pairs next to each other:
+//   2-D   W(l, j)    at j + KP l          (stage 1 writes pairs along j)
+//   3-D   T(i, j, k) at k + KP i + JS j   (stage A: pairs along k; stage B rewrites
+//                                          its fibers in place)
 // and the last stage writes pairs along i.
-template <typename S, int N, int D>
+// PART 0 is the first contraction, PART 1 the others (the kernel has a barrier and the
+// next tile's copies between them, once for all classes: the bodies of the classes
+// together are what the instruction cache has to hold).
+template <typename S, int N, int D, int PART>
 __device__ __forceinline__ void vl_tile(const VarlenArgs& a, int4 td, unsigned char* xt, float* ex1, const int* xo,
                                         const int* yo) {
-    constexpr int KP = vl_kp(N);
+    constexpr int KP = vl_kp(N), JS = vl_js(N);
     constexpr int R = vl_rows(N) / 2;
-    constexpr int EXQ = vl_e1_floats(D, N, (int)sizeof(S));   // exchange stride per instance (floats)
+    constexpr int EXQ = vl_e1_floats(D, N);                   // exchange stride per instance (floats)
     constexpr int SLOT = vl_xs_bytes(D, N, (int)sizeof(S));   // operand stride per instance (bytes)
     const float* m1 = a.coef + vl_slot(D, N);
     const float* m2 = m1 + vl_rows(N) * N;
@@ -245,8 +247,8 @@ __device__ __forceinline__ void vl_tile(const VarlenArgs& a, int4 td, unsigned c
     const int tid = threadIdx.x;
     const void* X = a.X;
     const void* Y = a.Y;
-    if constexpr (D == 2) {
-        const int F = cnt * N;
+    const int F = cnt * (D == 2 ? N : N * N);
+    if constexpr (D == 2 && PART == 0) {
         for (int f = tid; f < F; f += kVlThreads) {   // stage 1: mode 2, fibers (l, q)
             const int q = f / N, l = f - q * N;
             const S* xr = reinterpret_cast<const S*>(xt + q * SLOT) + vl_phase<S>(X, xo[q]) + l;
@@ -257,7 +259,7 @@ __device__ __forceinline__ void vl_tile(const VarlenArgs& a, int4 td, unsigned c
             vl_contract<N>(m2, x, w);
             vl_store_pairs<N>(ex1 + q * EXQ + KP * l, w);
         }
-        __syncthreads();
+    } else if constexpr (D == 2) {
         for (int f = tid; f < F; f += kVlThreads) {   // stage 2: mode 1, fibers (j, q)
             const int q = f / N, j = f - q * N;
             const float* wr = ex1 + q * EXQ + j;
@@ -268,181 +270,248 @@ __device__ __forceinline__ void vl_tile(const VarlenArgs& a, int4 td, unsigned c
             vl_contract<N>(m1, w, y);
             vl_stage_out<S, N>(reinterpret_cast<S*>(xt + q * SLOT) + vl_phase<S>(Y, yo[q]) + N * j, y);
         }
-    } else {
-        const int F = cnt * N * N;
+    } else if constexpr (PART == 0) {
         for (int f = tid; f < F; f += kVlThreads) {   // stage A: mode 3, fibers (i, j)
             const int q = f / (N * N), r = f - q * (N * N);
             const int i = r % N, j = r / N;
-            const S* xr = reinterpret_cast<const S*>(xt + q * SLOT) + vl_phase<S>(X, xo[q]) + i + N * j;
+            const S* xr = reinterpret_cast<const S*>(xt + q * SLOT) + vl_phase<S>(X, xo[q]) + r;
             float x[N];
 #pragma unroll
             for (int p = 0; p < N; ++p) x[p] = load_cvt<float, S>(xr[N * N * p]);
             f2 t[R];
             vl_contract<N>(m3, x, t);
-            vl_store_pairs<N>(ex1 + q * EXQ + KP * i + KP * N * j, t);
+            vl_store_pairs<N>(ex1 + q * EXQ + KP * i + JS * j, t);
         }
-        __syncthreads();
-        for (int f = tid; f < F; f += kVlThreads) {   // stage B: mode 2, fibers (i, k)
+    } else {
+        for (int f = tid; f < F; f += kVlThreads) {   // stage B: mode 2, fibers (i, k), in place
             const int q = f / (N * N), r = f - q * (N * N);
             const int k = r % N, i = r / N;
-            const float* tr = ex1 + q * EXQ + k + KP * i;
+            float* tr = ex1 + q * EXQ + k + KP * i;
             float t[N];
 #pragma unroll
-            for (int m = 0; m < N; ++m) t[m] = tr[KP * N * m];
+            for (int m = 0; m < N; ++m) t[m] = tr[JS * m];
             f2 u[R];
             vl_contract<N>(m2, t, u);
-            vl_store_pairs<N>(reinterpret_cast<float*>(xt + q * SLOT) + KP * k + KP * N * i, u);
+#pragma unroll
+            for (int m = 0; m < N; ++m) tr[JS * m] = (m & 1) ? f2_hi(u[m / 2]) : f2_lo(u[m / 2]);
         }
         __syncthreads();
         for (int f = tid; f < F; f += kVlThreads) {   // stage C: mode 1, fibers (j, k)
             const int q = f / (N * N), r = f - q * (N * N);
             const int j = r % N, k = r / N;
-            const float* ur = reinterpret_cast<const float*>(xt + q * SLOT) + j + KP * k;
+            const float* ur = ex1 + q * EXQ + k + JS * j;
             float u[N];
 #pragma unroll
-            for (int l = 0; l < N; ++l) u[l] = ur[KP * N * l];
+            for (int l = 0; l < N; ++l) u[l] = ur[KP * l];
             f2 y[R];
             vl_contract<N>(m1, u, y);
-            vl_stage_out<S, N>(reinterpret_cast<S*>(ex1 + q * EXQ) + vl_phase<S>(Y, yo[q]) + N * (j + N * k), y);
+            vl_stage_out<S, N>(reinterpret_cast<S*>(xt + q * SLOT) + vl_phase<S>(Y, yo[q]) + N * r, y);
         }
     }
 }
 
-template <typename S, int D>
-__device__ __forceinline__ void vl_dispatch_n(const VarlenArgs& a, int4 td, unsigned char* xt, float* ex1,
-                                              const int* xo, const int* yo) {
-    switch ((td.x & 15) + 1) {
-        case 1: vl_tile<S, 1, D>(a, td, xt, ex1, xo, yo); break;
-        case 2: vl_tile<S, 2, D>(a, td, xt, ex1, xo, yo); break;
-        case 3: vl_tile<S, 3, D>(a, td, xt, ex1, xo, yo); break;
-        case 4: vl_tile<S, 4, D>(a, td, xt, ex1, xo, yo); break;
-        case 5: vl_tile<S, 5, D>(a, td, xt, ex1, xo, yo); break;
-        case 6: vl_tile<S, 6, D>(a, td, xt, ex1, xo, yo); break;
-        case 7: vl_tile<S, 7, D>(a, td, xt, ex1, xo, yo); break;
-        case 8: vl_tile<S, 8, D>(a, td, xt, ex1, xo, yo); break;
-        case 9: vl_tile<S, 9, D>(a, td, xt, ex1, xo, yo); break;
-        case 10: vl_tile<S, 10, D>(a, td, xt, ex1, xo, yo); break;
-        case 11: vl_tile<S, 11, D>(a, td, xt, ex1, xo, yo); break;
-        case 12: vl_tile<S, 12, D>(a, td, xt, ex1, xo, yo); break;
-        case 13: vl_tile<S, 13, D>(a, td, xt, ex1, xo, yo); break;
-        case 14: vl_tile<S, 14, D>(a, td, xt, ex1, xo, yo); break;
-        case 15: vl_tile<S, 15, D>(a, td, xt, ex1, xo, yo); break;
-        case 16: vl_tile<S, 16, D>(a, td, xt, ex1, xo, yo); break;
+template <typename S, int PART>
+__device__ __forceinline__ void vl_dispatch(const VarlenArgs& a, int4 td, unsigned char* xt, float* ex1, const int* xo,
+                                            const int* yo) {
+    switch (td.x) {
+        case 0: vl_tile<S, 1, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 1: vl_tile<S, 2, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 2: vl_tile<S, 3, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 3: vl_tile<S, 4, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 4: vl_tile<S, 5, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 5: vl_tile<S, 6, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 6: vl_tile<S, 7, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 7: vl_tile<S, 8, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 8: vl_tile<S, 9, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 9: vl_tile<S, 10, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 10: vl_tile<S, 11, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 11: vl_tile<S, 12, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 12: vl_tile<S, 13, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 13: vl_tile<S, 14, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 14: vl_tile<S, 15, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 15: vl_tile<S, 16, 2, PART>(a, td, xt, ex1, xo, yo); break;
+        case 16: vl_tile<S, 1, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 17: vl_tile<S, 2, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 18: vl_tile<S, 3, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 19: vl_tile<S, 4, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 20: vl_tile<S, 5, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 21: vl_tile<S, 6, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 22: vl_tile<S, 7, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 23: vl_tile<S, 8, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 24: vl_tile<S, 9, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 25: vl_tile<S, 10, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 26: vl_tile<S, 11, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 27: vl_tile<S, 12, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 28: vl_tile<S, 13, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 29: vl_tile<S, 14, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 30: vl_tile<S, 15, 3, PART>(a, td, xt, ex1, xo, yo); break;
+        case 31: vl_tile<S, 16, 3, PART>(a, td, xt, ex1, xo, yo); break;
     }
 }
 
+// Work stealing by cluster launch control: asks the hardware to hand over a CTA of this
+// grid that has not started; the 16-byte answer lands in *res and completes on *bar.
+__device__ __forceinline__ void clc_request(uint4* res, uint64_t* bar) {
+    fence_proxy_async_smem();   // this thread's reads of the previous answer come first
+    mbar_arrive_expect_tx(bar, 16);
+    asm volatile(
+        "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+            smem_u32(res)),
+        "r"(smem_u32(bar))
+        : "memory");
+}
+// The index of the CTA handed over, or -1 if none was left.
+__device__ __forceinline__ int clc_answer(const uint4* res) {
+    unsigned got, x;
+    asm volatile(
+        "{\n\t.reg .b128 h;\n\t.reg .pred p;\n\t.reg .b32 y, z, w;\n\t"
+        "ld.shared.b128 h, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "mov.u32 %1, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, y, z, w}, h;\n\t}"
+        : "=r"(got), "=r"(x)
+        : "r"(smem_u32(res))
+        : "memory");
+    return got ? (int)x : -1;
+}
+
+// One CTA per tile is launched, but a running CTA keeps taking over the next one that has
+// not started, so that the grid is persistent and the tiles are still taken in the order
+// of the list, class by class: CTAs that walked fixed shares of it drifted apart until
+// every class's code ran at once and missed the instruction cache (the default workload:
+// 494 us; taken in order 379).
 template <typename S>
-__global__ void __launch_bounds__(kVlThreads, 3) varlen_kernel(const __grid_constant__ VarlenArgs a, int xbuf_bytes) {
+__global__ void __launch_bounds__(kVlThreads, 4) varlen_kernel(const __grid_constant__ VarlenArgs a, int xbuf_bytes) {
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);   // one barrier per operand buffer
+    uint64_t* clc_bar = full + 2;
+    uint4* clc_res = reinterpret_cast<uint4*>(smem + 32);
+    int* clc_next = reinterpret_cast<int*>(smem + 48);
     // Offsets of the instances of three consecutive tiles of this CTA (a ring):
-    // X offsets then Y offsets, kVlThreads each (a tile has at most that many).
+    // X offsets then Y offsets, kVlMaxP each.
     int* ring = reinterpret_cast<int*>(smem + 128);
-    unsigned char* xbuf = smem + 128 + 6 * kVlThreads * sizeof(int);
+    unsigned char* xbuf = smem + 128 + 6 * kVlMaxP * sizeof(int);
     float* ex1 = reinterpret_cast<float*>(xbuf + 2 * xbuf_bytes);
-    const int G = gridDim.x;
     const int tid = threadIdx.x;
-    const int t0 = blockIdx.x;
-    if (t0 >= a.ntiles) return;
     const int4 none = make_int4(0, 0, 0, 0);
+    if ((int)blockIdx.x >= a.ntiles) return;
+    // Thread 0 asks for tiles: one request at a time, none after the first refusal.  A grid
+    // smaller than the list walks it in fixed steps instead.
+    const bool steal = (int)gridDim.x == a.ntiles;
+    unsigned clc_phase = 0;
+    bool more = true;
+    int walk = blockIdx.x;
+    auto ask = [&]() {
+        if (steal && more) clc_request(clc_res, clc_bar);
+    };
+    auto take = [&]() -> int {   // the answer to the request in flight: a tile, or -1
+        if (!more) return -1;
+        int t = -1;
+        if (steal) {
+            if (mbar_wait_bounded(clc_bar, clc_phase, a.err)) t = clc_answer(clc_res);
+            clc_phase ^= 1u;
+        } else if ((walk += gridDim.x) < a.ntiles) {
+            t = walk;
+        }
+        more = t >= 0;
+        return t;
+    };
     if (tid == 0) {
         mbar_init(&full[0], 1);
         mbar_init(&full[1], 1);
+        mbar_init(clc_bar, 1);
         fence_barrier_init();
+        ask();
     }
-    // Pipeline: descriptors are read two tiles ahead, instance offsets one tile
-    // ahead (through the ring), operands one tile ahead (the other buffer).
-    int4 d0 = a.tiles[t0];
-    int4 d1 = t0 + G < a.ntiles ? a.tiles[t0 + G] : none;
-    int4 d2 = t0 + 2 * G < a.ntiles ? a.tiles[t0 + 2 * G] : none;
+    // Pipeline: tile numbers come two tiles ahead, descriptors and instance offsets during
+    // the tile before (offsets through the ring), operands one tile ahead (the other buffer).
+    int4 d0 = a.tiles[blockIdx.x];
     if (tid < d0.z) {
         ring[tid] = (int)a.xoff[d0.y + tid];
-        ring[kVlThreads + tid] = (int)a.yoff[d0.y + tid];
-    }
-    if (tid < d1.z) {
-        ring[2 * kVlThreads + tid] = (int)a.xoff[d1.y + tid];
-        ring[3 * kVlThreads + tid] = (int)a.yoff[d1.y + tid];
+        ring[kVlMaxP + tid] = (int)a.yoff[d0.y + tid];
     }
     __syncthreads();
     const uint64_t pol = l2_evict_first_policy();
-    int it = 0;
-    for (int tile = t0; tile < a.ntiles; ++it, tile += G) {
+    if (tid < 32) vl_issue_loads<S>(a, d0, ring, xbuf, &full[0], pol);
+    if (tid == 0) {
+        clc_next[0] = take();
+        ask();
+        clc_next[1] = take();
+    }
+    __syncthreads();
+    int4 d1 = clc_next[0] >= 0 ? a.tiles[clc_next[0]] : none;
+    int i2 = clc_next[1];
+    if (tid < d1.z) {
+        ring[2 * kVlMaxP + tid] = (int)a.xoff[d1.y + tid];
+        ring[3 * kVlMaxP + tid] = (int)a.yoff[d1.y + tid];
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int it = 0;; ++it) {
         const int b = it & 1;
         const int s0 = it % 3, s1 = (it + 1) % 3, s2 = (it + 2) % 3;
-        // offsets of tile + 2G, stored at the end of this tile
+        if (tid == 0) ask();
+        const int4 d2 = i2 >= 0 ? a.tiles[i2] : none;
+        const int key = d0.x;
+        unsigned char* xt = xbuf + b * xbuf_bytes;
+        const int* xo = ring + 2 * kVlMaxP * s0;
+        const int* yo = xo + kVlMaxP;
+        const bool ok = mbar_wait_bounded(&full[b], (unsigned)(it >> 1) & 1u, a.err);
+        vl_dispatch<S, 0>(a, d0, xt, ex1, xo, yo);
+        // A barrier, on which the CTA agrees whether the operands came; then warp 0 sends
+        // for the next tile's.  Their buffer holds the previous tile's results, whose stores
+        // were issued before this tile's first contraction: the wait for them is short.
+        if (__syncthreads_or(!ok)) {
+            // wait (bounded) for what is still in flight into this CTA's shared memory
+            if (tid == 0) {
+                mbar_wait_bounded(&full[b], (unsigned)(it >> 1) & 1u, a.err);
+                take();
+            }
+            if (tid < 32) bulk_wait_all();
+            return;
+        }
+        if (tid < 32 && d1.z) {
+            bulk_wait_read();
+            __syncwarp();
+            vl_issue_loads<S>(a, d1, ring + 2 * kVlMaxP * s1, xbuf + (b ^ 1) * xbuf_bytes, &full[b ^ 1], pol);
+        }
+        // offsets of the tile after next, stored at the end of this tile
         int xo2 = 0, yo2 = 0;
         if (tid < d2.z) {
             xo2 = (int)a.xoff[d2.y + tid];
             yo2 = (int)a.yoff[d2.y + tid];
         }
-        const int4 d3 = tile + 3 * G < a.ntiles ? a.tiles[tile + 3 * G] : none;
-        if (tid < 32) {
-            // The previous tile's results have left shared memory (the other operand
-            // buffer or the exchange buffer) before either is written again; then the
-            // operands of this tile (first iteration only) and of the next one.
-            bulk_wait_read();
-            __syncwarp();
-            for (int u = it == 0 ? 0 : 1; u < 2; ++u) {
-                const int4 du = u ? d1 : d0;
-                if (!du.z) break;
-                vl_issue_loads<S>(a, du, ring + 2 * kVlThreads * (u ? s1 : s0), xbuf + (b ^ u) * xbuf_bytes,
-                                  &full[b ^ u], pol);
-            }
-        }
-        const bool ok = mbar_wait_bounded(&full[b], (unsigned)(it >> 1) & 1u, a.err);
-        if (__syncthreads_or(!ok)) {
-            // wait (bounded) for copies still in flight into this CTA's buffers
-            if (tid == 0) {
-                mbar_wait_bounded(&full[b], (unsigned)(it >> 1) & 1u, a.err);
-                if (d1.z) mbar_wait_bounded(&full[b ^ 1], (unsigned)((it + 1) >> 1) & 1u, a.err);
-            }
-            if (tid < 32) bulk_wait_all();
-            return;
-        }
-        const int key = d0.x;
-        const int n = (key & 15) + 1;
-        unsigned char* xt = xbuf + b * xbuf_bytes;
-        const int* xo = ring + 2 * kVlThreads * s0;
-        const int* yo = xo + kVlThreads;
-        if (key < 16)
-            vl_dispatch_n<S, 2>(a, d0, xt, ex1, xo, yo);
-        else
-            vl_dispatch_n<S, 3>(a, d0, xt, ex1, xo, yo);
+        vl_dispatch<S, 1>(a, d0, xt, ex1, xo, yo);
         if (!a.alpha_one || !a.beta_zero) {
             // Epilogue Y = alpha (K x) + beta Y on the staged results (a separate pass,
             // so the contraction bodies stay as small as without it).  The values are
             // the storage-rounded results: for 16-bit storage this rounds twice.
             __syncthreads();
             const int nx = vl_nx(key);
-            const int slot = key < 16 ? vl_xs_bytes(2, n, (int)sizeof(S)) : 4 * vl_e1_floats(3, n, (int)sizeof(S));
-            unsigned char* base = key < 16 ? xt : reinterpret_cast<unsigned char*>(ex1);
+            const int slot = vl_xs_bytes(key < 16 ? 2 : 3, (key & 15) + 1, (int)sizeof(S));
             const S* Yg = static_cast<const S*>(a.Y);
             for (int e = tid; e < d0.z * nx; e += kVlThreads) {
                 const int q = e / nx, r = e - q * nx;
-                S* v = reinterpret_cast<S*>(base + q * slot) + vl_phase<S>(a.Y, yo[q]) + r;
+                S* v = reinterpret_cast<S*>(xt + q * slot) + vl_phase<S>(a.Y, yo[q]) + r;
                 float o = load_cvt<float, S>(*v);
                 if (!a.alpha_one) o *= a.alpha;
                 if (!a.beta_zero) o = __fmaf_rn(a.beta, load_cvt<float, S>(Yg[yo[q] + r]), o);
                 *v = store_cvt<S, float>(o);
             }
         }
+        if (tid < d2.z) {
+            ring[2 * kVlMaxP * s2 + tid] = xo2;
+            ring[2 * kVlMaxP * s2 + kVlMaxP + tid] = yo2;
+        }
+        if (tid == 0) clc_next[0] = take();
         fence_proxy_async_smem();   // results visible to the bulk copies
         __syncthreads();
-        if (tid < 32) {
-            if (key < 16)
-                vl_issue_stores<S>(a, d0, yo, xt, vl_xs_bytes(2, n, (int)sizeof(S)));
-            else
-                vl_issue_stores<S>(a, d0, yo, reinterpret_cast<const unsigned char*>(ex1),
-                                   4 * vl_e1_floats(3, n, (int)sizeof(S)));
-        }
-        if (tid < d2.z) {
-            ring[2 * kVlThreads * s2 + tid] = xo2;
-            ring[2 * kVlThreads * s2 + kVlThreads + tid] = yo2;
-        }
-        __syncthreads();
+        i2 = clc_next[0];
+        if (tid < 32) vl_issue_stores<S>(a, d0, yo, xt, vl_xs_bytes(key < 16 ? 2 : 3, (key & 15) + 1, (int)sizeof(S)));
         d0 = d1;
         d1 = d2;
-        d2 = d3;
+        if (!d0.z) break;
     }
     if (tid < 32) bulk_wait_all();
 }
@@ -450,20 +519,22 @@ __global__ void __launch_bounds__(kVlThreads, 3) varlen_kernel(const __grid_cons
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-// Largest tile of class (kind, n) whose operand and exchange buffers stay within
-// `budget` bytes each.
-static int vl_max_P(int kind, int n, size_t es, int budget) {
-    const int xs = vl_xs_bytes(kind, n, (int)es), ex = 4 * vl_e1_floats(kind, n, (int)es);
-    return std::max(1, std::min(kVlThreads, budget / std::max(xs, ex)));
+// Largest tile of class (kind, n) within the budgets of an operand buffer and of the
+// exchange buffer.
+static int vl_max_P(int kind, int n, size_t es, int xbudget, int ebudget) {
+    const int xs = vl_xs_bytes(kind, n, (int)es), ex = 4 * vl_e1_floats(kind, n);
+    return std::max(1, std::min(kVlMaxP, std::min(xbudget / xs, ebudget / ex)));
 }
 
-// Default tile, within the default buffer budget: as many instances as one
-// round of fibers (one per thread) covers in 2-D, two rounds in 3-D (the
-// tuner's choice on the mixed batch for most 3-D sizes: a second round halves
-// the share of the barrier waits).
-static int vl_default_P(int kind, int n, size_t es) {
-    const int fibers = kind == 2 ? kVlThreads / n : 2 * kVlThreads / (n * n);
-    return std::max(1, std::min(fibers, vl_max_P(kind, n, es, kVlBufBytes)));
+// Default tile of a class with `count` instances, within the default buffer budgets: as
+// many as two rounds of fibers (one per thread) cover in 3-D (a second round halves the
+// share of the barrier waits).  In 2-D one round, or two where the class then still has
+// two tiles for each of four CTAs on 152 SMs (n = 6, 833,333 instances: 163 -> 135 us;
+// in the mixed batch of 200,000 two rounds measured 1% slower).
+static int vl_default_P(int kind, int n, size_t es, int64_t count) {
+    auto fit = [&](int fibers) { return std::max(1, std::min(fibers, vl_max_P(kind, n, es, kVlXBytes, kVlEBytes))); };
+    const int two = fit(2 * kVlThreads / (kind == 2 ? n : n * n));
+    return kind == 3 || count >= (int64_t)2 * 4 * 152 * two ? two : fit(kVlThreads / n);
 }
 
 }  // namespace kron
@@ -510,6 +581,24 @@ static void* vl_kernel_ptr(kron_dtype io) {
     }
 }
 
+// CTAs of the launch.  Code of many large classes (a class's is about 24 bytes times
+// kind n^2) wants the tiles taken in order: one CTA per tile, running CTAs take over the
+// rest.  Below about 17 KB the instruction cache holds all of it, and short tiles are
+// 3-5% faster walked in fixed steps by the resident CTAs (3-D n = 16 alone: 90 us walked,
+// 86 taken in order; n = 6 alone: 68 and 70).
+static int vl_grid(const kron_varlen_plan* p, const void* fn, const DeviceInfo& dev) {
+    int units = 0;
+    for (int key = 0; key < kVlKeys; ++key) {
+        const int n = (key & 15) + 1;
+        if (p->present[key]) units += (key < 16 ? 2 : 3) * n * n;
+    }
+    const int tiles = (int)p->tiles.size();
+    if (units >= 700) return tiles;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kVlThreads, p->smem) != cudaSuccess) return 0;
+    return std::min(std::max(1, per_sm) * dev.sms, tiles);
+}
+
 // Sort by class, cut tiles, order them largest work first, size the workspace and smem.
 static kron_status vl_build(kron_varlen_plan* p) {
     const size_t es = elem_size(p->io);
@@ -533,13 +622,13 @@ static kron_status vl_build(kron_varlen_plan* p) {
             tl.push_back(T{flops * c, make_int4(key, (int)(start + s), c, 0)});
         }
         max_x = std::max(max_x, (size_t)P * vl_xs_bytes(kind, n, (int)es));
-        max_smem_rest = std::max(max_smem_rest, (size_t)P * vl_e1_floats(kind, n, (int)es) * sizeof(float));
+        max_smem_rest = std::max(max_smem_rest, (size_t)P * vl_e1_floats(kind, n) * sizeof(float));
     }
     if (p->order.size() > (size_t)INT32_MAX) return KRON_ERR_NOT_SUPPORTED;
     std::stable_sort(tl.begin(), tl.end(), [](const T& a, const T& b) { return a.work > b.work; });
     for (const T& t : tl) p->tiles.push_back(t.td);
     p->xbuf_bytes = (int)round_up(max_x, 128);
-    p->smem = 128 + 6 * kVlThreads * sizeof(int) + 2 * (size_t)p->xbuf_bytes + max_smem_rest;
+    p->smem = 128 + 6 * kVlMaxP * sizeof(int) + 2 * (size_t)p->xbuf_bytes + max_smem_rest;
     // Sized for one tile per instance (the most any tile size can give), so that
     // re-tuning never outgrows a workspace sized before it.
     p->ws_bytes = round_up(p->order.size() * sizeof(int4), 256) + 2 * round_up(p->order.size() * 8, 256);
@@ -609,11 +698,8 @@ static kron_status vl_launch(kron_varlen_plan* p, const void* X, void* Y, void* 
     }
     kron_status r = vl_fill_args(p, X, Y, ws);
     if (r != KRON_OK) return r;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kVlThreads, p->smem) != cudaSuccess)
-        return KRON_ERR_CUDA;
-    int grid = std::max(1, per_sm) * dev.sms;
-    grid = (int)std::min<size_t>((size_t)grid, p->tiles.size());
+    const int grid = vl_grid(p, fn, dev);
+    if (grid < 1) return KRON_ERR_CUDA;
     int xbe = p->xbuf_bytes;
     void* kargs[2] = {p->args, &xbe};
     cudaKernelNodeParams kp = {};
@@ -699,8 +785,7 @@ KRON_API kron_status kron_varlen_plan_create(kron_varlen_plan** plan, int num_cl
         }
         int tp = 0, td = 0;
         kron_get_tile_config(d.kind, n, io, (kron_compute)kVarlenTag, &tp, &td);
-        p->P[key] = (tp > 0 && tp <= vl_max_P(d.kind, n, elem_size(io), kVlMaxBufBytes)) ? tp
-                                                                                     : vl_default_P(d.kind, n, elem_size(io));
+        p->P[key] = (tp > 0 && tp <= vl_max_P(d.kind, n, elem_size(io), kVlMaxBufBytes, kVlMaxBufBytes)) ? tp : 0;
     }
     p->cls_of.resize(batch_count);
     p->xoff.assign(h_x_off, h_x_off + batch_count);
@@ -719,6 +804,11 @@ KRON_API kron_status kron_varlen_plan_create(kron_varlen_plan** plan, int num_cl
         xt = std::max(xt, h_x_off[i] + nx);
         yt = std::max(yt, h_y_off[i] + nx);
     }
+    int64_t count[kVlKeys] = {};
+    for (int64_t i = 0; i < batch_count; ++i) count[p->cls_of[i]]++;
+    for (int key = 0; key < kVlKeys; ++key)
+        if (p->present[key] && p->P[key] == 0)
+            p->P[key] = vl_default_P(key < 16 ? 2 : 3, (key & 15) + 1, elem_size(io), count[key]);
     // Instances of Y must not overlap (each output element written once).
     {
         std::vector<std::pair<int64_t, int64_t>> r(batch_count);
@@ -816,7 +906,7 @@ KRON_API kron_status kron_varlen_tune(kron_varlen_plan* plan, const void* X, voi
     for (size_t w = 0; w < work.size() && st == KRON_OK; ++w) {
         const int key = work[w].second;
         const int kind = key < 16 ? 2 : 3, n = (key & 15) + 1;
-        const int pmax = vl_max_P(kind, n, elem_size(plan->io), kVlMaxBufBytes);
+        const int pmax = vl_max_P(kind, n, elem_size(plan->io), kVlMaxBufBytes, kVlMaxBufBytes);
         const int cur = plan->P[key];
         int best_P = cur;
         // Besides the neighbours of the current tile: the tile whose fibers per stage
@@ -899,11 +989,8 @@ KRON_API kron_status kron_varlen_execute_noalloc(kron_varlen_plan* plan, const v
     if (r != KRON_OK) return r;
     void* fn = vl_kernel_ptr(plan->io);
     if (!ensure_smem_optin(fn, plan->smem)) return KRON_ERR_CUDA;   // the attribute only ever grows
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kVlThreads, plan->smem) != cudaSuccess)
-        return KRON_ERR_CUDA;
-    int grid = std::max(1, per_sm) * dev.sms;
-    grid = (int)std::min<size_t>((size_t)grid, plan->tiles.size());
+    const int grid = vl_grid(plan, fn, dev);
+    if (grid < 1) return KRON_ERR_CUDA;
     int xbe = plan->xbuf_bytes;
     void* kargs[2] = {plan->args, &xbe};
     if (cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kVlThreads), kargs, plan->smem, st) != cudaSuccess)
