@@ -161,6 +161,46 @@ KRON_API kron_status kron3_batched(kron_stream_t stream, char transa, char trans
                                    kron_compute comp);
 
 /*
+ * kron2_batched_args, kron3_batched_args -- the same calls with all arguments but the
+ * components in one structure, for language bindings whose cost grows with the number of
+ * arguments.
+ * alpha and beta are given as (re, im) in double precision and rounded to the type the
+ * storage wants (im is read for complex storage only).  The structure is read during the
+ * call.  Results and errors are those of kron2_batched / kron3_batched;
+ * KRON_ERR_INVALID_VALUE for a null pointer.
+ */
+typedef struct {
+    kron_stream_t stream;
+    int64_t batch_count;
+    const void* X;
+    void* Y;
+    int64_t ldxp, ldyp;
+    double alpha_re, alpha_im, beta_re, beta_im;
+    int ma, na, mb, nb;
+    int lda, ldb, ldx, ldy;
+    kron_dtype io;
+    kron_compute comp;
+    char transa, transb, transx;
+} kron2_args;
+
+typedef struct {
+    kron_stream_t stream;
+    int64_t batch_count;
+    const void* X;
+    void* Y;
+    int64_t ldxp, ldyp;
+    double alpha_re, alpha_im, beta_re, beta_im;
+    int ma, na, mb, nb, mc, nc;
+    int lda, ldb, ldc, ldx, ldx2, ldy, ldy2;
+    kron_dtype io;
+    kron_compute comp;
+    char transa, transb, transc;
+} kron3_args;
+
+KRON_API kron_status kron2_batched_args(const kron2_args* args, const void* A, const void* B);
+KRON_API kron_status kron3_batched_args(const kron3_args* args, const void* A, const void* B, const void* C);
+
+/*
  * kron1_batched -- the paper's TKRON1 (Sec. 3), the 1-D product ("almost a
  * batched GEMV"):
  *

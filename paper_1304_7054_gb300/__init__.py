@@ -15,6 +15,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -37,6 +38,8 @@ SIGNATURES = {
                        _I, _I], _I),
     "kron3_batched": ([_P, _C, _C, _C, _I, _I, _I, _I, _I, _I, _L, _P, _P, _I, _P, _I, _P, _I, _P, _I, _I,
                        _L, _P, _P, _I, _I, _L, _I, _I], _I),
+    "kron2_batched_args": ([_P, _P, _P], _I),
+    "kron3_batched_args": ([_P, _P, _P, _P], _I),
     "kron1_batched": ([_P, _C, _I, _I, _L, _P, _P, _I, _P, _L, _P, _P, _L, _I, _I], _I),
     "kron_gemm_a_batched": ([_P, _C, _C, _I, _I, _I, _P, _P, _I, _L, _P, _I, _P, _P, _I, _L, _L, _I, _I, _I],
                             _I),
@@ -97,19 +100,35 @@ def _torch():
     return torch
 
 
+_io_codes = None   # torch dtype -> storage code
+
+
 def _io_of(t) -> int:
-    torch = _torch()
-    m = {torch.float32: "f32", torch.float64: "f64", torch.bfloat16: "bf16", torch.float16: "f16",
-         torch.complex64: "c64", torch.complex128: "c128"}
-    if t.dtype not in m:
+    global _io_codes
+    if _io_codes is None:
+        torch = _torch()
+        m = {torch.float32: "f32", torch.float64: "f64", torch.bfloat16: "bf16", torch.float16: "f16",
+             torch.complex64: "c64", torch.complex128: "c128"}
+        _io_codes = {k: DTYPES[v] for k, v in m.items()}
+    code = _io_codes.get(t.dtype)
+    if code is None:
         raise TypeError(f"unsupported storage dtype {t.dtype}")
-    return DTYPES[m[t.dtype]]
+    return code
+
+
+_raw_stream = None   # the current stream's handle, by the shortest way this torch has
 
 
 def _stream_handle(stream) -> int:
-    torch = _torch()
+    global _raw_stream
     if stream is None:
-        stream = torch.cuda.current_stream()
+        if _raw_stream is None:
+            torch = _torch()
+            torch.cuda.current_stream()   # initialises CUDA
+            get, dev = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+            _raw_stream = (lambda: get(dev())) if get and dev else (
+                lambda: torch.cuda.current_stream().cuda_stream)
+        return _raw_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -122,6 +141,27 @@ def _comp_buffer(M, ctype):
     if M.ndim == 2:
         return np.ascontiguousarray(M.T).ravel(), M.shape[0]
     return np.ascontiguousarray(M.ravel()), None
+
+
+def _comp_bytes(M, ctype):
+    """As _comp_buffer, as a bytes object (kept alive by the caller during the call)."""
+    if type(M) is np.ndarray and M.dtype == ctype and M.ndim == 2:
+        return M.tobytes("F"), M.shape[0]
+    buf, ld = _comp_buffer(M, ctype)
+    return buf.tobytes(), ld
+
+
+# kron2_args and kron3_args of kron.h in native layout.
+_ARGS2 = struct.Struct("@PqPPqqdddd4i4iiiccc5x")
+_ARGS3 = struct.Struct("@PqPPqqdddd6i7iiiccc1x")
+
+
+def _re_im(v, ctype):
+    """A host scalar as (re, im); im = 0 for real compute types."""
+    if ctype is np.complex64 or ctype is np.complex128:
+        v = complex(v)
+        return v.real, v.imag
+    return (v if type(v) is float else ctypes.c_double(v).value), 0.0
 
 
 def _device_operand(t, need, name):
@@ -143,9 +183,12 @@ def _scalar(v, ctype):
     return (ctypes.c_double if ctype == np.float64 else ctypes.c_float)(v)
 
 
+_CTYPES = {DTYPES["f64"]: np.float64, DTYPES["c64"]: np.complex64, DTYPES["c128"]: np.complex128}
+
+
 def _ctype_of(io):
     """Host type of the components, alpha and beta for storage type io."""
-    return {DTYPES["f64"]: np.float64, DTYPES["c64"]: np.complex64, DTYPES["c128"]: np.complex128}.get(io, np.float32)
+    return _CTYPES.get(io, np.float32)
 
 
 def kron2_batched(A, B, X, Y, *, ma, na, mb, nb, batch, alpha=1.0, beta=0.0, transa="N", transb="N",
@@ -153,13 +196,13 @@ def kron2_batched(A, B, X, Y, *, ma, na, mb, nb, batch, alpha=1.0, beta=0.0, tra
                   compute="native", stream=None):
     """Y^p <- alpha op(B) op(X^p) op(A)^T + beta Y^p on CUDA tensors X, Y (storage
     f32/f64/bf16/f16, flat column-major instances); A, B host arrays."""
-    L = load_library()
+    L = _lib or load_library()
     io = _io_of(X)
-    if _io_of(Y) != io:
+    if Y.dtype is not X.dtype and _io_of(Y) != io:
         raise TypeError("X and Y must have the same dtype")
     ctype = _ctype_of(io)
-    Ab, lda0 = _comp_buffer(A, ctype)
-    Bb, ldb0 = _comp_buffer(B, ctype)
+    Ab, lda0 = _comp_bytes(A, ctype)
+    Bb, ldb0 = _comp_bytes(B, ctype)
     ta, tb, tx = transa.upper(), transb.upper(), transx.upper()
     lda = lda or lda0 or (ma if ta == "N" else na)
     ldb = ldb or ldb0 or (mb if tb == "N" else nb)
@@ -167,14 +210,21 @@ def kron2_batched(A, B, X, Y, *, ma, na, mb, nb, batch, alpha=1.0, beta=0.0, tra
     ldxp = ldx * (na if tx == "N" else nb) if ldxp is None else ldxp
     ldy = ldy or mb
     ldyp = ldy * ma if ldyp is None else ldyp
-    al, be = _scalar(alpha, ctype), _scalar(beta, ctype)
     xr, xc = (nb, na) if tx == "N" else (na, nb)
     xp = _device_operand(X, (batch - 1) * ldxp + ldx * (xc - 1) + xr if batch > 0 else 0, "X")
     yp = _device_operand(Y, (batch - 1) * ldyp + ldy * (ma - 1) + mb if batch > 0 else 0, "Y")
-    st = L.kron2_batched(_stream_handle(stream), ta.encode(), tb.encode(), tx.encode(), ma, na, mb, nb, batch,
-                         ctypes.addressof(al), Ab.ctypes.data, lda, Bb.ctypes.data, ldb, xp, ldx, ldxp,
-                         ctypes.addressof(be), yp, ldy, ldyp, io, COMPUTE[compute])
-    _check(st, "kron2_batched")
+    s, comp = _stream_handle(stream), COMPUTE[compute]
+    try:
+        args = _ARGS2.pack(s, batch, xp, yp, ldxp, ldyp, *_re_im(alpha, ctype), *_re_im(beta, ctype), ma, na, mb, nb,
+                           lda, ldb, ldx, ldy, io, comp, ta.encode(), tb.encode(), tx.encode())
+    except struct.error:   # not representable: the argument-by-argument call says what is wrong
+        al, be = _scalar(alpha, ctype), _scalar(beta, ctype)
+        st = L.kron2_batched(s, ta.encode(), tb.encode(), tx.encode(), ma, na, mb, nb, batch, ctypes.addressof(al), Ab,
+                             lda, Bb, ldb, xp, ldx, ldxp, ctypes.addressof(be), yp, ldy, ldyp, io, comp)
+    else:
+        st = L.kron2_batched_args(args, Ab, Bb)
+    if st != KRON_OK:
+        raise KronError(st, "kron2_batched")
     return Y
 
 
@@ -182,14 +232,14 @@ def kron3_batched(A, B, C, X, Y, *, ma, na, mb, nb, mc, nc, batch, alpha=1.0, be
                   transb="N", transc="N", lda=None, ldb=None, ldc=None, ldx=None, ldx2=None, ldxp=None,
                   ldy=None, ldy2=None, ldyp=None, compute="native", stream=None):
     """Y^p <- alpha (op(A) (x) op(B) (x) op(C)) vec(X^p) + beta Y^p (C on mode 1)."""
-    L = load_library()
+    L = _lib or load_library()
     io = _io_of(X)
-    if _io_of(Y) != io:
+    if Y.dtype is not X.dtype and _io_of(Y) != io:
         raise TypeError("X and Y must have the same dtype")
     ctype = _ctype_of(io)
-    Ab, lda0 = _comp_buffer(A, ctype)
-    Bb, ldb0 = _comp_buffer(B, ctype)
-    Cb, ldc0 = _comp_buffer(C, ctype)
+    Ab, lda0 = _comp_bytes(A, ctype)
+    Bb, ldb0 = _comp_bytes(B, ctype)
+    Cb, ldc0 = _comp_bytes(C, ctype)
     ta, tb, tc = transa.upper(), transb.upper(), transc.upper()
     lda = lda or lda0 or (ma if ta == "N" else na)
     ldb = ldb or ldb0 or (mb if tb == "N" else nb)
@@ -200,21 +250,29 @@ def kron3_batched(A, B, C, X, Y, *, ma, na, mb, nb, mc, nc, batch, alpha=1.0, be
     ldy = ldy or mc
     ldy2 = ldy2 or ldy * mb
     ldyp = ldy2 * ma if ldyp is None else ldyp
-    al, be = _scalar(alpha, ctype), _scalar(beta, ctype)
     xp = _device_operand(X, (batch - 1) * ldxp + ldx2 * (na - 1) + ldx * (nb - 1) + nc if batch > 0 else 0, "X")
     yp = _device_operand(Y, (batch - 1) * ldyp + ldy2 * (ma - 1) + ldy * (mb - 1) + mc if batch > 0 else 0, "Y")
-    st = L.kron3_batched(_stream_handle(stream), ta.encode(), tb.encode(), tc.encode(), ma, na, mb, nb, mc, nc,
-                         batch, ctypes.addressof(al), Ab.ctypes.data, lda, Bb.ctypes.data, ldb, Cb.ctypes.data,
-                         ldc, xp, ldx, ldx2, ldxp, ctypes.addressof(be), yp, ldy, ldy2, ldyp,
-                         io, COMPUTE[compute])
-    _check(st, "kron3_batched")
+    s, comp = _stream_handle(stream), COMPUTE[compute]
+    try:
+        args = _ARGS3.pack(s, batch, xp, yp, ldxp, ldyp, *_re_im(alpha, ctype), *_re_im(beta, ctype), ma, na, mb, nb,
+                           mc, nc, lda, ldb, ldc, ldx, ldx2, ldy, ldy2, io, comp, ta.encode(), tb.encode(),
+                           tc.encode())
+    except struct.error:   # not representable: the argument-by-argument call says what is wrong
+        al, be = _scalar(alpha, ctype), _scalar(beta, ctype)
+        st = L.kron3_batched(s, ta.encode(), tb.encode(), tc.encode(), ma, na, mb, nb, mc, nc, batch,
+                             ctypes.addressof(al), Ab, lda, Bb, ldb, Cb, ldc, xp, ldx, ldx2, ldxp,
+                             ctypes.addressof(be), yp, ldy, ldy2, ldyp, io, comp)
+    else:
+        st = L.kron3_batched_args(args, Ab, Bb, Cb)
+    if st != KRON_OK:
+        raise KronError(st, "kron3_batched")
     return Y
 
 
 def kron1_batched(A, X, Y, *, ma, na, batch, alpha=1.0, beta=0.0, transa="N", lda=None, ldxp=None, ldyp=None,
                   compute="native", stream=None):
     """TKRON1: y^p <- alpha op(A) x^p + beta y^p on CUDA tensors X, Y; A a host array."""
-    L = load_library()
+    L = _lib or load_library()
     io = _io_of(X)
     if _io_of(Y) != io:
         raise TypeError("X and Y must have the same dtype")

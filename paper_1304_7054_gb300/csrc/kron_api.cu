@@ -6,6 +6,7 @@
 #include <atomic>
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <utility>
 
 #include "kron_device.cuh"
@@ -64,6 +65,25 @@ bool ensure_smem_optin(const void* fn, size_t bytes) {
     if (bytes <= cur) return true;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
     cur = bytes;
+    return true;
+}
+
+bool resident_ctas(int* per_sm, const void* fn, int threads, size_t smem) {
+    typedef std::tuple<const void*, int, int, size_t> Key;
+    static std::map<Key, int> known;
+    static std::mutex mu;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    const Key key(fn, dev, threads, smem);
+    auto it = known.find(key);
+    if (it == known.end()) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem) != cudaSuccess) return false;
+        if (known.size() >= 4096) known.clear();   // mixed-size plans bring sizes of their own
+        it = known.emplace(key, n).first;
+    }
+    *per_sm = it->second;
     return true;
 }
 
@@ -359,8 +379,7 @@ KRON_API kron_status kron2_batched(kron_stream_t stream, char transa, char trans
     if (ranges_overlap(X, xbytes, Y, ybytes)) return KRON_ERR_ALIAS;
     if ((st = device_range(X, xbytes)) != KRON_OK || (st = device_range(Y, ybytes)) != KRON_OK) return st;
 
-    static thread_local KronDesc d;
-    d = KronDesc();
+    KronDesc d;
     const bool dbl = io == KRON_R64F || io == KRON_C64F;
     d.D = 2;
     d.N = std::max(std::max(ma, na), std::max(mb, nb));
@@ -371,7 +390,6 @@ KRON_API kron_status kron2_batched(kron_stream_t stream, char transa, char trans
         op_pad(d.m1, d.N, B, ldb, tb, mb, nb, dbl);
         op_pad(d.m2, d.N, A, lda, ta, ma, na, dbl);
     }
-    memset(d.m3, 0, sizeof(d.m3));
     d.X = X;
     d.Y = Y;
     d.batch = batch_count;
@@ -395,6 +413,32 @@ KRON_API kron_status kron2_batched(kron_stream_t stream, char transa, char trans
     d.ycontig = d.contiguous && ldy == N && ldyp == (int64_t)N * N && ((uintptr_t)Y) % 16 == 0;
     choose_yvec(d);
     return dispatch(d, (cudaStream_t)stream);
+}
+
+// The scalar (re, im) in the type of alpha and beta for storage io.
+struct HostScalar {
+    double v[2];
+    HostScalar(double re, double im, kron_dtype io) {
+        const double d[2] = {re, im};
+        const float f[2] = {(float)re, (float)im};
+        if (io == KRON_R64F || io == KRON_C64F) memcpy(v, d, sizeof(d));
+        else memcpy(v, f, sizeof(f));
+    }
+};
+
+KRON_API kron_status kron2_batched_args(const kron2_args* a, const void* A, const void* B) {
+    if (!a) return KRON_ERR_INVALID_VALUE;
+    const HostScalar al(a->alpha_re, a->alpha_im, a->io), be(a->beta_re, a->beta_im, a->io);
+    return kron2_batched(a->stream, a->transa, a->transb, a->transx, a->ma, a->na, a->mb, a->nb, a->batch_count, al.v,
+                         A, a->lda, B, a->ldb, a->X, a->ldx, a->ldxp, be.v, a->Y, a->ldy, a->ldyp, a->io, a->comp);
+}
+
+KRON_API kron_status kron3_batched_args(const kron3_args* a, const void* A, const void* B, const void* C) {
+    if (!a) return KRON_ERR_INVALID_VALUE;
+    const HostScalar al(a->alpha_re, a->alpha_im, a->io), be(a->beta_re, a->beta_im, a->io);
+    return kron3_batched(a->stream, a->transa, a->transb, a->transc, a->ma, a->na, a->mb, a->nb, a->mc, a->nc,
+                         a->batch_count, al.v, A, a->lda, B, a->ldb, C, a->ldc, a->X, a->ldx, a->ldx2,
+                         a->ldxp, be.v, a->Y, a->ldy, a->ldy2, a->ldyp, a->io, a->comp);
 }
 
 static double host_scalar(const void* v, kron_dtype io) {
@@ -527,8 +571,7 @@ KRON_API kron_status kron3_batched(kron_stream_t stream, char transa, char trans
     if (ranges_overlap(X, xbytes, Y, ybytes)) return KRON_ERR_ALIAS;
     if ((st = device_range(X, xbytes)) != KRON_OK || (st = device_range(Y, ybytes)) != KRON_OK) return st;
 
-    static thread_local KronDesc d;
-    d = KronDesc();
+    KronDesc d;
     const bool dbl = io == KRON_R64F || io == KRON_C64F;
     d.D = 3;
     d.N = std::max(std::max(std::max(ma, na), std::max(mb, nb)), std::max(mc, nc));

@@ -589,7 +589,7 @@ kron_status launch_fiber_n(const KronDesc& d, cudaStream_t st) {
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFiberThreads, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, kFiberThreads, smem))
             return KRON_ERR_CUDA;
         if (per_sm < 1) per_sm = 1;
         grid = (int64_t)per_sm * dev.sms;

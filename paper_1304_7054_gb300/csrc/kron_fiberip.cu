@@ -263,7 +263,7 @@ kron_status launch_fi_n(const KronDesc& d, cudaStream_t st) {
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFiCompute * G + 32, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, kFiCompute * G + 32, smem))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }

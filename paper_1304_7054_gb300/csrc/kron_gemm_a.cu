@@ -187,7 +187,7 @@ kron_status launch_ga_pair(const GemmADesc& g, cudaStream_t st) {
     int64_t grid = g.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGaThreads, 0) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, kGaThreads, 0))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }
@@ -343,7 +343,7 @@ kron_status launch_ga_tma(const GemmADesc& g, cudaStream_t st) {
     int64_t grid = g.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGaThreads, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, kGaThreads, smem))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }
@@ -437,7 +437,7 @@ kron_status launch_ga(const GemmADesc& g, Kern kern, cudaStream_t st) {
     int64_t grid = g.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGaThreads, 0) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, kGaThreads, 0))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }

@@ -18,13 +18,14 @@ constexpr int kFiberThreads = 256;   // threads per CTA of the CUDA-core kernels
 struct KronDesc {
     int D = 2;          // 2 or 3
     int N = 1;          // padded size, 1..16
+    // (the N x N entries in use are written by the caller: m3 in 3-D only, the imaginary
+    // parts for complex storage only)
     double m1[kMaxN * kMaxN];
     double m2[kMaxN * kMaxN];
     double m3[kMaxN * kMaxN];
-    // imaginary parts (complex storage; zero otherwise)
-    double m1i[kMaxN * kMaxN] = {};
-    double m2i[kMaxN * kMaxN] = {};
-    double m3i[kMaxN * kMaxN] = {};
+    double m1i[kMaxN * kMaxN];
+    double m2i[kMaxN * kMaxN];
+    double m3i[kMaxN * kMaxN];
     const void* X = nullptr;
     void* Y = nullptr;
     int64_t batch = 0, ldxp = 0, ldyp = 0;
@@ -155,5 +156,10 @@ const DeviceInfo& device_info();
 // Raises the dynamic shared-memory limit of kernel `fn` on the current device to
 // at least `bytes` (remembered per kernel and device).  False on a CUDA error.
 bool ensure_smem_optin(const void* fn, size_t bytes);
+
+// CTAs of kernel `fn` that an SM of the current device holds at this launch shape (the
+// occupancy query costs about as much as the launch, so its answers are remembered).
+// False on a CUDA error.
+bool resident_ctas(int* per_sm, const void* fn, int threads, size_t smem);
 
 }  // namespace kron

@@ -330,8 +330,7 @@ kron_status launch_k1(const GemmADesc& g, cudaStream_t st) {
                 const void* kern = (const void*)kron1t_kernel;
                 if (!ensure_smem_optin(kern, smem)) return KRON_ERR_CUDA;
                 int per_sm = 0;
-                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kron1t_kernel, kK1Threads, smem) !=
-                    cudaSuccess)
+                if (!resident_ctas(&per_sm, (const void*)kron1t_kernel, kK1Threads, smem))
                     return KRON_ERR_CUDA;
                 const int64_t ntiles = (g.batch + TV - 1) / TV;
                 int64_t grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
@@ -347,7 +346,7 @@ kron_status launch_k1(const GemmADesc& g, cudaStream_t st) {
     const size_t smem = (size_t)kK1Warps * 2 * 32 * N * sizeof(S);
     if (!ensure_smem_optin((const void*)kern, smem)) return KRON_ERR_CUDA;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kK1Threads, smem) != cudaSuccess)
+    if (!resident_ctas(&per_sm, (const void*)kern, kK1Threads, smem))
         return KRON_ERR_CUDA;
     const int64_t chunks = (g.batch + 31) / 32;
     int64_t grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;

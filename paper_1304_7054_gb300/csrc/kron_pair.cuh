@@ -476,7 +476,7 @@ kron_status launch_pair_n(const KronDesc& d, cudaStream_t st) {
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem) != cudaSuccess) return KRON_ERR_CUDA;
+        if (!resident_ctas(&per_sm, (const void*)kern, NT, smem)) return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }
     if (grid > ntiles) grid = ntiles;

@@ -618,7 +618,7 @@ kron_status launch_pair16(const KronDesc& d, cudaStream_t st) {
             int64_t grid = d.grid;
             if (grid <= 0) {
                 int per_sm = 0;
-                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess)
+                if (!resident_ctas(&per_sm, (const void*)kern, threads, smem))
                     return KRON_ERR_CUDA;
                 grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
             }
@@ -651,7 +651,7 @@ kron_status launch_pair16(const KronDesc& d, cudaStream_t st) {
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, kThreads, smem))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }

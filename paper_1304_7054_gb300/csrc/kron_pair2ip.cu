@@ -254,7 +254,7 @@ kron_status launch_ip_n(const KronDesc& d, cudaStream_t st) {
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, threads, smem))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }

@@ -366,7 +366,7 @@ kron_status launch_pk_n(const KronDesc& d, cudaStream_t st) {
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, kThreads, smem))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }
@@ -420,7 +420,7 @@ kron_status launch_pair3ip(const KronDesc& d, cudaStream_t st) {
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair3ip_kernel, kThreads, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)pair3ip_kernel, kThreads, smem))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }

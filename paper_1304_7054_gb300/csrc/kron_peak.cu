@@ -83,7 +83,7 @@ extern "C" KRON_API kron_status kron_peak_probe(kron_stream_t stream, int unit, 
     const void* fn = unit == 0 ? (const void*)peak_ffma2_kernel
                    : unit == 1 ? (const void*)peak_ffma_kernel : (const void*)peak_dfma_kernel;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kPeakThreads, 0) != cudaSuccess || per_sm < 1)
+    if (!resident_ctas(&per_sm, (const void*)fn, kPeakThreads, 0) || per_sm < 1)
         return KRON_ERR_CUDA;
     const int grid = per_sm * dev.sms;
     // a = 1 - 2^-20 and b = 2^-30 keep every chain finite and away from the sink value

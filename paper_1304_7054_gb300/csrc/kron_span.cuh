@@ -486,7 +486,7 @@ kron_status launch_span_n(const KronDesc& d, const SpanArgs& a, size_t smem, cud
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSpanThreads, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, kSpanThreads, smem))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }

@@ -1526,7 +1526,7 @@ static kron_status launch_tc2_n(const KronDesc& d, cudaStream_t st) {
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTcThreads, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, kTcThreads, smem))
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }
@@ -1579,7 +1579,7 @@ static kron_status launch_tc3_n(const KronDesc& d, cudaStream_t st) {
         auto kern = tc3g_kernel<S, N>;
         if (!ensure_smem_optin((const void*)kern, smem)) return KRON_ERR_CUDA;
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * W, smem) != cudaSuccess)
+        if (!resident_ctas(&per_sm, (const void*)kern, 32 * W, smem))
             return KRON_ERR_CUDA;
         int64_t grid = d.grid > 0 ? d.grid : (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
         if (grid > d.batch) grid = d.batch;
@@ -1592,7 +1592,7 @@ static kron_status launch_tc3_n(const KronDesc& d, cudaStream_t st) {
     auto kern = tc3_kernel<S, N>;
     if (!ensure_smem_optin((const void*)kern, smem)) return KRON_ERR_CUDA;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTc3Warps, smem) != cudaSuccess)
+    if (!resident_ctas(&per_sm, (const void*)kern, 32 * kTc3Warps, smem))
         return KRON_ERR_CUDA;
     int64_t grid = d.grid > 0 ? d.grid : (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     const int64_t need = (d.batch + kTc3Warps - 1) / kTc3Warps;

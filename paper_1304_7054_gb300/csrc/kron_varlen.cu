@@ -595,7 +595,7 @@ static int vl_grid(const kron_varlen_plan* p, const void* fn, const DeviceInfo& 
     const int tiles = (int)p->tiles.size();
     if (units >= 700) return tiles;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kVlThreads, p->smem) != cudaSuccess) return 0;
+    if (!resident_ctas(&per_sm, (const void*)fn, kVlThreads, p->smem)) return 0;
     return std::min(std::max(1, per_sm) * dev.sms, tiles);
 }
 
