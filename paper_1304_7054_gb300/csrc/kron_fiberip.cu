@@ -43,7 +43,7 @@ struct FiberIpArgs {
     void* Y;
     int64_t batch;
     int P, nstage;
-    int beta_zero, alpha_one;
+    int alpha_one;
     float alpha, beta;
     unsigned* err;
 };
@@ -75,7 +75,8 @@ __device__ __forceinline__ void fiber_in_place(float* p, const f2* Mp) {
     for (int r = 0; r < N; ++r) p[S * r] = (r & 1) ? f2_hi(y[r / 2]) : f2_lo(y[r / 2]);
 }
 
-template <int N, int D>
+// YB: beta != 0; the old results come in by bulk copy too.
+template <int N, int D, bool YB>
 __global__ void __launch_bounds__(fi_max_threads<D>(), fi_min_blocks<D>())
 fiberip_kernel(const __grid_constant__ FiberIpArgs<N> a, int G) {
     constexpr int NN = N * N, NX = D == 3 ? NN * N : NN;
@@ -86,6 +87,7 @@ fiberip_kernel(const __grid_constant__ FiberIpArgs<N> a, int G) {
     float* ring = reinterpret_cast<float*>(smem + 256);
     const int NB = a.nstage, P = a.P;
     const int tile_words = P * NX;
+    const int slot_words = YB ? 2 * tile_words : tile_words;   // operands, then old results
     const int ncompute = kFiCompute * G;
     const int gidx = threadIdx.x / kFiCompute;
     const int tid = threadIdx.x - kFiCompute * gidx;   // thread within its compute group
@@ -111,7 +113,7 @@ fiberip_kernel(const __grid_constant__ FiberIpArgs<N> a, int G) {
             // whole 16-byte chunks by bulk copy; a ragged last tile's tail is
             // stored by the compute threads
             const unsigned bytes = ((unsigned)c * NX * 4u) & ~15u;
-            if (lane == 0 && bytes) bulk_s2g_hint(Y + i0 * NX, ring + s * tile_words, bytes, pol);
+            if (lane == 0 && bytes) bulk_s2g_hint(Y + i0 * NX, ring + s * slot_words, bytes, pol);
             bulk_commit();
         };
         int it = 0;
@@ -130,8 +132,9 @@ fiberip_kernel(const __grid_constant__ FiberIpArgs<N> a, int G) {
             const unsigned bytes = ((unsigned)cnt * NX * 4u) & ~15u;   // the compute threads load the rest
             fence_proxy_async_smem();
             if (lane == 0) {
-                mbar_arrive_expect_tx(&full[s], bytes);
-                if (bytes) bulk_g2s(ring + s * tile_words, X + i0 * NX, bytes, &full[s], pol);
+                mbar_arrive_expect_tx(&full[s], YB ? 2 * bytes : bytes);
+                if (bytes) bulk_g2s(ring + s * slot_words, X + i0 * NX, bytes, &full[s], pol);
+                if (bytes && YB) bulk_g2s(ring + s * slot_words + tile_words, Y + i0 * NX, bytes, &full[s], pol);
             }
         }
         for (int j = it > NB ? it - NB : 0; j < it; ++j) {
@@ -147,13 +150,16 @@ fiberip_kernel(const __grid_constant__ FiberIpArgs<N> a, int G) {
     for (int it = gidx; blockIdx.x + (int64_t)it * grid < ntiles; it += G) {
         const int64_t tile = blockIdx.x + (int64_t)it * grid;
         const int s = it % NB;
-        float* buf = ring + s * tile_words;
+        float* buf = ring + s * slot_words;
         const int64_t i0 = tile * P;
         const int cnt = (int)min((int64_t)P, a.batch - i0);
         const int nel = cnt * NX, nbulk = (int)((((unsigned)nel * 4u) & ~15u) / 4u);
         const bool ok = mbar_wait_bounded(&full[s], (unsigned)(it / NB) & 1u, a.err);
         if (nbulk != nel) {   // ragged last tile: the elements past the last 16-byte chunk
-            for (int e = nbulk + tid; e < nel; e += kFiCompute) buf[e] = X[i0 * NX + e];
+            for (int e = nbulk + tid; e < nel; e += kFiCompute) {
+                buf[e] = X[i0 * NX + e];
+                if (YB) buf[tile_words + e] = Y[i0 * NX + e];
+            }
             group_sync_or(false, gidx);
         }
         if constexpr (D == 3) {
@@ -189,12 +195,11 @@ fiberip_kernel(const __grid_constant__ FiberIpArgs<N> a, int G) {
             for (int l = 0; l < N; ++l) x[l] = p[l];
             f2 y[(N + 1) / 2];
             contract_pairs<N>(a.m1, x, y);
-            const float* yg = Y + (i0 + q) * NX + N * r;
 #pragma unroll
             for (int i = 0; i < N; ++i) {
                 float v = (i & 1) ? f2_hi(y[i / 2]) : f2_lo(y[i / 2]);
                 if (!a.alpha_one) v *= a.alpha;
-                if (!a.beta_zero) v = fmaf(a.beta, yg[i], v);
+                if (YB) v = fmaf(a.beta, p[tile_words + i], v);
                 p[i] = v;
             }
         }
@@ -237,7 +242,6 @@ kron_status launch_fi_n(const KronDesc& d, cudaStream_t st) {
     a.batch = d.batch;
     a.alpha = (float)d.alpha;
     a.beta = (float)d.beta;
-    a.beta_zero = d.beta == 0.0;
     a.alpha_one = d.alpha == 1.0;
     a.err = device_error_word();
     if (!a.err) return KRON_ERR_CUDA;
@@ -252,12 +256,17 @@ kron_status launch_fi_n(const KronDesc& d, cudaStream_t st) {
     int nb = d.nstage >= 1 ? d.nstage : 2 * G;
     if (nb > kFiMaxRing) nb = kFiMaxRing;
     nb = nb < G ? G : nb / G * G;
-    auto smem_of = [&](int n_b) { return 256 + (size_t)n_b * a.P * NX * sizeof(float); };
+    // With beta != 0 the old results come in by bulk copy beside the operands (read from
+    // global memory by the threads of a stage, n words apart, they cost n = 9 a quarter of
+    // its time: 188 -> 146 us): a ring of the same bytes holds half the tiles.
+    const bool yb = d.beta != 0.0;
+    if (yb && d.nstage < 1) nb = std::max(G, nb / 2 / G * G);
+    auto smem_of = [&](int n_b) { return 256 + (size_t)n_b * a.P * NX * sizeof(float) * (yb ? 2 : 1); };
     size_t smem = smem_of(nb);
     while (nb > G && smem > dev.smem_per_block_optin) smem = smem_of(nb -= G);
     if (smem > dev.smem_per_block_optin) return KRON_ERR_NOT_SUPPORTED;
     a.nstage = nb;
-    auto kern = fiberip_kernel<N, D>;
+    auto kern = yb ? fiberip_kernel<N, D, true> : fiberip_kernel<N, D, false>;
     if (!ensure_smem_optin((const void*)kern, smem)) return KRON_ERR_CUDA;
     const int64_t ntiles = (d.batch + a.P - 1) / a.P;
     int64_t grid = d.grid;

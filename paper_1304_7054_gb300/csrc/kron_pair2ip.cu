@@ -18,9 +18,9 @@
 //    instances times 2 adjacent units (row pairs in the first stage, columns
 //    in the second), so the eight-byte shared accesses of a half-warp cover
 //    the 32 banks once: no bank conflicts.
-//  * One producer warp streams tiles in and results out through a ring of
-//    buffers (full / empty mbarriers); the four compute warps issue no global
-//    memory access except the reads of Y that beta != 0 needs.
+//  * One producer warp streams tiles in (with beta != 0 their old results too) and
+//    results out through a ring of buffers (full / empty mbarriers); the compute warps
+//    issue no global memory access.
 #include "kron_pair.cuh"
 
 namespace kron {
@@ -61,7 +61,8 @@ __device__ __forceinline__ void load_col(const float* p, float (&w)[N]) {
 // A CTA holds G compute groups of four warps and one producer warp; group g
 // takes the CTA's tiles it = g mod G from one shared ring, so one CTA per SM
 // can keep a deep ring in flight while its groups work.
-template <int N>
+// YB: beta != 0; the old results come in by bulk copy too.
+template <int N, bool YB>
 __global__ void __launch_bounds__(kIpCompute * kIpMaxGroups + 32, 1) pair2ip_kernel(const __grid_constant__ PairArgs<N, 2> a,
                                                                                      int G) {
     using L = IpLayout<N>;
@@ -73,6 +74,7 @@ __global__ void __launch_bounds__(kIpCompute * kIpMaxGroups + 32, 1) pair2ip_ker
     const int P = a.P;             // a multiple of 8
     const int QG = P >> 3;
     const int tile_words = P * L::NX;
+    const int slot_words = YB ? 2 * tile_words : tile_words;   // operands, then old results
     const int ncompute = kIpCompute * G;
     const int gidx = threadIdx.x / kIpCompute;
     const int tid = threadIdx.x - kIpCompute * gidx;   // thread within its group (producer: lane + 128)
@@ -99,7 +101,7 @@ __global__ void __launch_bounds__(kIpCompute * kIpMaxGroups + 32, 1) pair2ip_ker
         auto store_tile = [&](int s, int64_t t) {
             const int64_t i0 = t * P;
             const int c = (int)min((int64_t)P, a.batch - i0);
-            if (lane == 0) bulk_s2g_hint(Y + i0 * L::NX, ring + s * tile_words, (unsigned)c * L::NX * 4u, pol);
+            if (lane == 0) bulk_s2g_hint(Y + i0 * L::NX, ring + s * slot_words, (unsigned)c * L::NX * 4u, pol);
             bulk_commit();
         };
         int it = 0;
@@ -115,13 +117,17 @@ __global__ void __launch_bounds__(kIpCompute * kIpMaxGroups + 32, 1) pair2ip_ker
             }
             const int64_t inst0 = tile * P;
             const int cnt = (int)min((int64_t)P, a.batch - inst0);
-            float* buf = ring + s * tile_words;
+            float* buf = ring + s * slot_words;
             // The compute threads' generic accesses to this buffer happen before their
             // arrival on empty[s]; order them before the bulk copies that overwrite it.
             fence_proxy_async_smem();
-            if (lane == 0) mbar_arrive_expect_tx(&full[s], (unsigned)cnt * L::NX * 4u);
+            const unsigned bytes = (unsigned)cnt * L::NX * 4u;
+            if (lane == 0) mbar_arrive_expect_tx(&full[s], YB ? 2 * bytes : bytes);
             __syncwarp();
-            if (lane == 0) bulk_g2s(buf, X + inst0 * L::NX, (unsigned)cnt * L::NX * 4u, &full[s], pol);
+            if (lane == 0) {
+                bulk_g2s(buf, X + inst0 * L::NX, bytes, &full[s], pol);
+                if (YB) bulk_g2s(buf + tile_words, Y + inst0 * L::NX, bytes, &full[s], pol);
+            }
         }
         for (int j = it > NB ? it - NB : 0; j < it; ++j) {   // the last tiles' results
             if (!mbar_wait_bounded(&empty[j % NB], (unsigned)(j / NB) & 1u, a.err)) break;
@@ -132,11 +138,10 @@ __global__ void __launch_bounds__(kIpCompute * kIpMaxGroups + 32, 1) pair2ip_ker
     }
 
     const f2* m1p = reinterpret_cast<const f2*>(a.m1);
-    const float* Y = static_cast<const float*>(a.Y);
     for (int it = gidx; blockIdx.x + (int64_t)it * grid < ntiles; it += G) {
         const int64_t tile = blockIdx.x + (int64_t)it * grid;
         const int s = it % NB;
-        float* buf = ring + s * tile_words;
+        float* buf = ring + s * slot_words;
         const int64_t inst0 = tile * P;
         const int cnt = (int)min((int64_t)P, a.batch - inst0);
         const bool ok = mbar_wait_bounded(&full[s], (unsigned)(it / NB) & 1u, a.err);
@@ -185,8 +190,8 @@ __global__ void __launch_bounds__(kIpCompute * kIpMaxGroups + 32, 1) pair2ip_ker
 #pragma unroll
                 for (int k = 0; k < N / 2; ++k) y[k] = fmul2(y[k], al);
             }
-            if (!a.beta_zero) {
-                const float* yq = Y + (inst0 + q) * L::NX + N * j;
+            if constexpr (YB) {
+                const float* yq = wq + tile_words;
                 const f2 be = f2_pack(a.beta, a.beta);
 #pragma unroll
                 for (int k = 0; k < N / 2; ++k) y[k] = ffma2(be, load_pair<float>(yq + 2 * k), y[k]);
@@ -200,8 +205,8 @@ __global__ void __launch_bounds__(kIpCompute * kIpMaxGroups + 32, 1) pair2ip_ker
 }
 
 template <int N>
-size_t ip_smem_bytes(int P, int nb) {
-    return 256 + (size_t)nb * P * IpLayout<N>::NX * sizeof(float);
+size_t ip_smem_bytes(int P, int nb, bool ybuf) {
+    return 256 + (size_t)nb * P * IpLayout<N>::NX * sizeof(float) * (ybuf ? 2 : 1);
 }
 
 template <int N>
@@ -242,12 +247,17 @@ kron_status launch_ip_n(const KronDesc& d, cudaStream_t st) {
     int nb = d.nstage >= 1 ? d.nstage : (d.warps > 0 || d.P > 0 ? 2 * G : L::NB0);
     if (nb > kIpMaxRing) nb = kIpMaxRing;
     nb = nb < G ? G : nb / G * G;
-    size_t smem = ip_smem_bytes<N>(P, nb);
-    while (nb > G && smem > dev.smem_per_block_optin) smem = ip_smem_bytes<N>(P, nb -= G);
+    // beta != 0: the old results come in beside the operands, so a ring of the same bytes
+    // holds half the tiles (60 M elements: n = 10 140 -> 111 us, n = 14 148 -> 122 us against
+    // reading them column by column from global memory).
+    const bool ybuf = !a.beta_zero;
+    if (ybuf && d.nstage < 1) nb = nb / 2 < G ? G : nb / 2 / G * G;
+    size_t smem = ip_smem_bytes<N>(P, nb, ybuf);
+    while (nb > G && smem > dev.smem_per_block_optin) smem = ip_smem_bytes<N>(P, nb -= G, ybuf);
     if (smem > dev.smem_per_block_optin) return KRON_ERR_NOT_SUPPORTED;
     a.P = P;
     a.nstage = nb;
-    auto kern = pair2ip_kernel<N>;
+    auto kern = ybuf ? pair2ip_kernel<N, true> : pair2ip_kernel<N, false>;
     if (!ensure_smem_optin((const void*)kern, smem)) return KRON_ERR_CUDA;
     const int threads = kIpCompute * G + 32;
     const int64_t ntiles = (d.batch + P - 1) / P;
