@@ -410,25 +410,35 @@ size_t pair_smem_bytes(int P, int nstage) {
     return 128 + nstage * round_up((size_t)P * L::SX * sizeof(S), 128) + (size_t)P * (L::EX1 + L::EX2) * sizeof(float);
 }
 
-// Default tile: threads per CTA and instances per tile for each (N, kind), and
-// fibers per step of the last contraction (two measured faster for 3-D n >= 14,
-// one elsewhere).
-template <int N, int D>
+// Default tile: threads per CTA, instances per tile, ring depth and fibers per step of the
+// last contraction for each (N, kind, storage size).
+//
+// FP32: two fibers per step measured faster for 3-D n >= 14, one elsewhere; one buffer in
+// flight gives the most resident CTAs, which matters more than a deeper ring.
+// 16-bit storage: two fibers per step for n = 4, 8, 16 (2-D n = 8: 75 -> 64 us for 60 M
+// elements with the second buffer; 3-D n = 8: 80 -> 75, n = 16: 127 -> 117; n = 14: 148 -> 158,
+// so not there); in 2-D a tile is half the bytes of an FP32 one, and twice the instances
+// pay up to n = 10 (n = 4: 78 -> 64 us with a second buffer, n = 6: 67 -> 62, n = 10:
+// 80 -> 67; n = 12: 70 -> 74; at n = 8 the second fiber already does it).  Only with
+// beta = 0: old values of Y read by more fibers at once cost more (n = 4: 86 -> 124 us).
+template <int N, int D, int SB>
 struct PairConfig {
     static constexpr int NT = 128;
-    static constexpr int FPS = (D == 3 && N >= 14) ? 2 : 1;
+    static constexpr bool POW2 = (N & (N - 1)) == 0;
+    static constexpr int FPS = SB == 2 ? (POW2 && N >= 4 ? 2 : 1) : (D == 3 && N >= 14 ? 2 : 1);
+    static constexpr int DEPTH = SB == 2 && D == 2 && POW2 ? 2 : 1;
     // about one unit of first-stage work per thread (3-D: rounded up, so that a
     // tile keeps every thread busy in the first stage, measured 1.2x faster at
     // n = 12 than rounding down to one instance; two units at n <= 8, where the
     // tuner's choices were 1.1x faster)
-    static constexpr int P0 = (D == 2) ? (2 * NT) / N
+    static constexpr int P0 = (D == 2) ? (SB == 2 && N <= 10 && N != 8 ? 2 : 1) * ((2 * NT) / N)
                                        : (N <= 8 ? 2 : 1) * ((2 * NT + N * N - 1) / (N * N));
 };
 
 template <typename S, int N, int D>
 kron_status launch_pair_n(const KronDesc& d, cudaStream_t st) {
     using L = PairLayout<N, D, (int)sizeof(S)>;
-    constexpr int NT = PairConfig<N, D>::NT;
+    constexpr int NT = PairConfig<N, D, (int)sizeof(S)>::NT;
     const DeviceInfo& dev = device_info();
     if (dev.sms <= 0) return KRON_ERR_CUDA;
     PairArgs<N, D> a;
@@ -454,22 +464,22 @@ kron_status launch_pair_n(const KronDesc& d, cudaStream_t st) {
     a.alpha_one = d.alpha == 1.0;
     a.err = device_error_word();
     if (!a.err) return KRON_ERR_CUDA;
-    int P = d.P > 0 ? d.P : PairConfig<N, D>::P0;
+    using Cfg = PairConfig<N, D, (int)sizeof(S)>;
+    const bool plain = sizeof(S) == 2 && D == 2 && d.beta != 0.0;   // the FP32 choices instead
+    int P = d.P > 0 ? d.P : (plain ? PairConfig<N, D, 4>::P0 : Cfg::P0);
     if (!L::XPAD) {
         int mult = 1;
         while ((mult * L::NX * sizeof(S)) % 16) ++mult;
         P = (P + mult - 1) / mult * mult;
     }
-    // One stage in flight gives the most resident CTAs, which matters more than a
-    // deeper pipeline (measured for both kinds).
-    int nstage = d.nstage >= 1 ? d.nstage : 1;
+    int nstage = d.nstage >= 1 ? d.nstage : (plain ? 1 : Cfg::DEPTH);
     if (nstage > 8) nstage = 8;
     size_t smem = pair_smem_bytes<S, N, D>(P, nstage);
     while (nstage > 1 && smem > dev.smem_per_block_optin) smem = pair_smem_bytes<S, N, D>(P, --nstage);
     if (smem > dev.smem_per_block_optin) return KRON_ERR_NOT_SUPPORTED;
     a.P = P;
     a.nstage = nstage;
-    const int fps = d.fps > 0 ? d.fps : PairConfig<N, D>::FPS;
+    const int fps = d.fps > 0 ? d.fps : (plain ? 1 : Cfg::FPS);
     auto kern = fps == 2 ? pair_kernel<S, N, D, NT, 2> : pair_kernel<S, N, D, NT, 1>;
     if (!ensure_smem_optin((const void*)kern, smem)) return KRON_ERR_CUDA;
     const int64_t ntiles = (d.batch + P - 1) / P;
