@@ -409,8 +409,7 @@ def measure_variant(kg, name, steps, warmup, torch, dev, peaks, tune=True):
     gbs = by / (kern_ms * 1e-3) / 1e9
     r = {"gflops": round(fl / (kern_ms * 1e-3) / 1e9, 1), "hbm_gbs": round(gbs, 1),
          "hbm_frac": round(gbs / peaks["hbm"], 4), "ms": round(kern_ms, 4), "batch": b.batch,
-         "kernel": kernel_of(b.kind, b.n, wl["io"], wl["compute"], (tile or {}).get("variant", "auto"),
-                             (tile or {}).get("compute_warps", 0)),
+         "kernel": dispatched_kernel(b.kind, b.n, wl["io"], wl["compute"], tile),
          "max_norm_err_vs_fp64_oracle": err,
          "tuned_config": tile}
     if wl["io"] in ("bf16", "f16"):
@@ -543,9 +542,24 @@ def measure_interfaces(kg, steps, warmup, torch, dev, peaks):
     return out
 
 
+def dispatched_kernel(kind, n, io, compute, tile):
+    """kernel_of for a contiguous batch with beta = 0 and the tuning table's entry `tile`
+    (None or all zero: the built-in choice), with the library's rule that split-precision
+    calls of small n run on the CUDA cores unless the table holds something for them."""
+    tile = tile or {}
+    untuned = tile.get("variant", "auto") == "auto" and not any(v for k, v in tile.items() if k != "variant")
+    small = (n <= (15 if kind == 2 else 14)) if io == "f32" else (
+        n <= 9 or n == 11 if kind == 2 else n <= 12)
+    if compute == "bf16x3" and untuned and small:
+        compute = "native"
+    if compute == "native" and untuned and io in ("bf16", "f16") and n % 2 == 1 and n > 1:
+        return f"span_kernel<{io},n={n},{kind}-D>"
+    return kernel_of(kind, n, io, compute, tile.get("variant", "auto"), tile.get("compute_warps", 0))
+
+
 def kernel_of(kind, n, io, compute, variant="auto", warps=0):
-    """Name of the kernel the library dispatches a contiguous batch to (with the
-    kernel body and compute warps the tuning table holds for it)."""
+    """Name of the kernel body of a contiguous batch's compute mode (with the body and
+    compute warps the tuning table holds for it)."""
     if compute == "bf16x3":
         if kind == 3 and (warps > 1 or (warps == 0 and (
                 (n >= 14 and not (io == "f16" and n != 16)) or (io == "f32" and n >= 10 and n % 2 == 0)))):
