@@ -162,10 +162,25 @@ __device__ __forceinline__ void span_contract(const f2* __restrict__ M, const fl
     }
 }
 
-// One stage over F fibers, two per thread and step.  in(f, x) reads fiber f and
-// returns where its outputs go; out(dst, o, y01, y23) writes rows o..o+3.
-template <int NI, typename In, typename Out>
+// Two fibers per thread and step, except with runtime extents above 8: there two of them
+// do not fit in the 128 registers that four CTAs per SM leave a thread (NI = 16: up to 1168
+// bytes of spill stores and 2496 of loads; one fiber: none, and calls of that body take
+// 0.43-1.0 of the time; NI = 4 and 8 have room for two, and one is up to 1.2x slower).
+template <int NI, int NO>
+constexpr bool span_two() { return NO > 0 || NI <= 8; }
+
+// One stage over F fibers.  in(f, x) reads fiber f and returns where its outputs go;
+// out(dst, o, y01, y23) writes rows o..o+3.
+template <int NI, int NO, typename In, typename Out>
 __device__ __forceinline__ void span_stage_run(const f2* M, int F, int rows, In in, Out out) {
+    if constexpr (!span_two<NI, NO>()) {
+        for (int f = threadIdx.x; f < F; f += kSpanThreads) {
+            float x[1][NI];
+            auto* d0 = in(f, x[0]);
+            span_contract<NI, 1>(M, x, rows, [&](int, int o, f2 y0, f2 y1) { out(d0, o, y0, y1); });
+        }
+        return;
+    }
     for (int f = threadIdx.x; f < F; f += 2 * kSpanThreads) {
         if (f + kSpanThreads < F) {
             float x[2][NI];
@@ -213,7 +228,7 @@ __device__ __forceinline__ void span_last(const SpanArgs& a, int F, const float*
     const f2 al = f2_pack(a.alpha, a.alpha);
     const int so = MODE == 2 ? a.so : 1, rows = sh.rows(L);
     const bool alpha_one = a.alpha_one;
-    span_stage_run<NI>(
+    span_stage_run<NI, NO>(
         a.m[L], F, rows,
         [&](int f, float (&x)[NI]) {
             const int q = sh.div_fib(L, f), r = f - q * sh.fib(L);
@@ -383,7 +398,7 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
         // ---- first contraction: operand span -> e -------------------------------------
         {
             const int rows = sh.rows(0), ldxq = (int)a.ldxp, col = a.xs_col;
-            span_stage_run<NI>(
+            span_stage_run<NI, NO>(
                 a.m[0], cnt * sh.fib(0), rows,
                 [&](int f, float (&x)[NI]) {
                     const int q = sh.div_fib(0, f), r = f - q * sh.fib(0);
@@ -424,7 +439,7 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
         // ---- 3-D second contraction, in place -----------------------------------------
         if constexpr (D == 3) {
             const int rows = sh.rows(1), js = sh.js();
-            span_stage_run<NI>(
+            span_stage_run<NI, NO>(
                 a.m[1], cnt * sh.fib(1), rows,
                 [&](int f, float (&x)[NI]) {
                     const int q = sh.div_fib(1, f), r = f - q * sh.fib(1);
