@@ -4,8 +4,11 @@
 // A general layout is still a run of memory per tile: the span from the first
 // element of a tile's first operand to the last element of its last one, padding
 // included, arrives as ONE bulk copy (TMA) into a ring of buffers and is addressed
-// in shared memory with the caller's own strides.  Padding inside a span costs
-// little: DRAM delivers whole 32-byte sectors anyway.  (The fiber kernel this
+// in shared memory with the caller's own strides.  A copy takes whole 16-byte granules; the
+// tiles at either end of X, where such a granule would hold bytes that are not X's, go to
+// CTAs of their own that load the elements there one by one (a test for them inside the tile
+// loop cost every shape 5-20%).  Padding inside a span costs little: DRAM delivers whole 32-byte
+// sectors anyway.  (The fiber kernel this
 // replaces loads each element with its own division and bounds test, with nothing
 // in flight behind the arithmetic; spans mostly made of gaps are left to it.)
 //
@@ -53,6 +56,7 @@
 #include <algorithm>
 
 #include "kron_pair.cuh"
+#include "kron_span_copy.h"
 
 namespace kron {
 
@@ -75,6 +79,7 @@ struct SpanArgs {
     int64_t batch, ldxp, ldyp;    // elements
     int xs_col, xs_plane;         // strides of the contracted / plane index of X (elements)
     int xspan;                    // elements spanned by one operand
+    int head, tail;               // first / last tiles whose copies would reach outside X
     int ce[3];                    // contracted extent of each stage
     int oe[3];                    // output extent of each stage
     int kp, js;                   // strides of the exchange buffer
@@ -363,6 +368,27 @@ __device__ __forceinline__ void span_issue(const SpanArgs& a, unsigned char* dst
     bulk_g2s(dst, (const void*)a0, bytes, bar, pol);
 }
 
+// As span_issue, for the whole CTA: the copy takes the granules that lie inside the span,
+// the threads load the elements before and after them.  The caller's barrier follows.
+template <typename S>
+__device__ __forceinline__ void span_issue_inside(const SpanArgs& a, unsigned char* dst, uint64_t* bar, int64_t tile,
+                                                  uint64_t pol) {
+    const int64_t inst0 = tile * a.P;
+    const int cnt = (int)min((int64_t)a.P, a.batch - inst0);
+    const uintptr_t b0 = (uintptr_t)(static_cast<const S*>(a.X) + inst0 * a.ldxp);
+    const uintptr_t b1 = b0 + ((cnt - 1) * a.ldxp + a.xspan) * sizeof(S);
+    const uintptr_t from = (b0 + 15) & ~(uintptr_t)15, to = b1 & ~(uintptr_t)15;
+    unsigned char* buf = dst - (b0 & ~(uintptr_t)15);   // + address
+    if (threadIdx.x == 0) {
+        const unsigned bytes = to > from ? (unsigned)(to - from) : 0u;
+        mbar_arrive_expect_tx(bar, bytes);
+        if (bytes) bulk_g2s(buf + from, (const void*)from, bytes, bar, pol);
+    }
+    const uintptr_t head = b0 + threadIdx.x * sizeof(S), tail = (to > from ? to : from) + threadIdx.x * sizeof(S);
+    if (head < from && head < b1) *reinterpret_cast<S*>(buf + head) = *reinterpret_cast<const S*>(head);
+    if (tail < b1) *reinterpret_cast<S*>(buf + tail) = *reinterpret_cast<const S*>(tail);
+}
+
 template <typename S, int NI, int NO, int D>
 __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_constant__ SpanArgs a) {
     const SpanShape<NI, NO, D> sh{a};
@@ -371,22 +397,32 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
     unsigned char* slots = smem + 128;
     float* e = reinterpret_cast<float*>(slots + kSpanRing * a.slot_bytes);
     const int tid = threadIdx.x;
-    const int64_t ntiles = (a.batch + a.P - 1) / a.P;
-    const int64_t grid = gridDim.x;
+    // The last CTAs of the grid take the tiles at the ends of X whose copies would reach
+    // outside, one each; the others walk the tiles between them.
+    const int walkers = (int)gridDim.x - a.head - a.tail;
+    const int grid = walkers > 0 ? walkers : 1;   // step of the walk
+    int64_t first = a.head + (int)blockIdx.x, end = (a.batch + a.P - 1) / a.P - a.tail;
+    const bool edge = (int)blockIdx.x >= walkers;
+    if (edge) {
+        first = (int)blockIdx.x - walkers;
+        if (first >= a.head) first += end - a.head;
+        end = first + 1;
+    }
     uint64_t pol = 0;
     if (tid == 0) {
         for (int s = 0; s < kSpanRing; ++s) mbar_init(&full[s], 1);
         fence_barrier_init();
         pol = l2_evict_first_policy();
         for (int s = 0; s < kSpanRing; ++s) {
-            const int64_t t = blockIdx.x + s * grid;
-            if (t < ntiles) span_issue<S>(a, slots + s * a.slot_bytes, &full[s], t, pol);
+            const int64_t t = first + s * grid;
+            if (t < end && !edge) span_issue<S>(a, slots + s * a.slot_bytes, &full[s], t, pol);
         }
     }
+    if (edge) span_issue_inside<S>(a, slots, full, first, pol);
     __syncthreads();
 
     int it = 0;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += grid, ++it) {
+    for (int64_t tile = first; tile < end; tile += grid, ++it) {
         const int s = it % kSpanRing;
         const int64_t inst0 = tile * a.P;
         const int cnt = (int)min((int64_t)a.P, a.batch - inst0);
@@ -420,7 +456,7 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {   // let in-flight copies land before the CTA exits
                 for (int j = it; j < it + kSpanRing - (it > 0); ++j)
-                    if (blockIdx.x + (int64_t)j * grid < ntiles)
+                    if (tile + (int64_t)(j - it) * grid < end)
                         mbar_wait_bounded(&full[j % kSpanRing], (unsigned)(j / kSpanRing) & 1u, a.err);
                 bulk_wait_all();
             }
@@ -429,7 +465,7 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
         // The previous tile's slot: its results have left, the next operands come in.
         if (tid == 0 && it > 0) {
             const int64_t next = tile + (kSpanRing - 1) * grid;
-            if (next < ntiles) {
+            if (next < end) {
                 const int p = (it - 1) % kSpanRing;
                 bulk_wait_read();
                 fence_proxy_async_smem();
@@ -497,7 +533,7 @@ kron_status launch_span_n(const KronDesc& d, const SpanArgs& a, size_t smem, cud
     const DeviceInfo& dev = device_info();
     auto kern = span_kernel<S, NI, NO, D>;
     if (!ensure_smem_optin((const void*)kern, smem)) return KRON_ERR_CUDA;
-    const int64_t ntiles = (d.batch + a.P - 1) / a.P;
+    const int64_t ntiles = (d.batch + a.P - 1) / a.P, edges = a.head + a.tail;
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
@@ -505,7 +541,8 @@ kron_status launch_span_n(const KronDesc& d, const SpanArgs& a, size_t smem, cud
             return KRON_ERR_CUDA;
         grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * dev.sms;
     }
-    grid = std::max<int64_t>(1, std::min<int64_t>(grid, ntiles));
+    // (one CTA for each tile that is loaded element by element, at least one for the rest)
+    grid = std::max<int64_t>(edges + (ntiles > edges), std::min<int64_t>(grid, ntiles));
     kern<<<(unsigned)grid, kSpanThreads, smem, st>>>(a);
     return cudaPeekAtLastError() == cudaSuccess ? KRON_OK : KRON_ERR_CUDA;
 }
@@ -668,6 +705,10 @@ kron_status launch_span(const KronDesc& d, cudaStream_t st) {
     while (smem > dev.smem_per_block_optin && P > 1) smem = smem_of(--P);
     if (smem > dev.smem_per_block_optin) return KRON_ERR_NOT_SUPPORTED;
     a.P = P;
+    const SpanEdges ed = span_edges((uintptr_t)d.X, d.batch, P, d.batch > 1 ? d.ldxp : 0, xspan, es);
+    if (!ed.copies) return KRON_ERR_NOT_SUPPORTED;
+    a.head = ed.head;
+    a.tail = ed.tail;
     {
         const int ch = y1 / a.vec;
         a.dc = kSpanThreads % ch;
