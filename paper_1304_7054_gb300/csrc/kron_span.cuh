@@ -57,6 +57,7 @@
 
 #include "kron_pair.cuh"
 #include "kron_span_copy.h"
+#include "kron_span_rule.h"
 
 namespace kron {
 
@@ -595,19 +596,25 @@ kron_status launch_span(const KronDesc& d, cudaStream_t st) {
     const int64_t useful = (int64_t)x1 * x2 * x3;
     // A span that is mostly gaps is read element by element instead (fiber kernel).
     if (xspan > 2 * useful || (d.batch > 1 && d.ldxp > 2 * useful)) return KRON_ERR_NOT_SUPPORTED;
-    // Where the fiber kernel measured faster (its speed over this one's): 1 x 1 components
-    // (1.05-1.25); in 3-D the row chunks of short rows with beta != 0 (n = 5: 1.09, n = 6:
-    // 1.03; n = 7: 0.86); 16-bit storage without an instantiation of its own, where n is
-    // even and large or the kind is 3-D (13 -> 14: 1.25 in 2-D and 1.47 in 3-D, 11 -> 12:
-    // 0.70 in 2-D; odd results, 12 -> 13: 0.46 and 0.85).
-    if (d.N == 1 || (D == 3 && d.beta != 0.0 && d.N <= 6)) return KRON_ERR_NOT_SUPPORTED;
     const bool square = x1 == d.N && x2 == d.N && (D == 2 || x3 == d.N) && d.ye[0] == d.N && d.ye[1] == d.N &&
                         (D == 2 || d.ye[2] == d.N);
-    if (es == 2 && !square && d.N % 2 == 0 && (D == 3 || d.N > 12)) return KRON_ERR_NOT_SUPPORTED;
-    // ... and large 3-D extents that differ per mode, which run with runtime bounds up to 16
-    // ((13,16,15) -> (16,13,14): 1.20 with padded strides; (12,12,12) -> (12,12,8): 0.56).
     const bool cubic = x1 == x2 && d.ye[0] == d.ye[1] && (D == 2 || (x1 == x3 && d.ye[0] == d.ye[2]));
-    if (D == 3 && !cubic && x1 + x2 + x3 + d.ye[0] + d.ye[1] + d.ye[2] > 76) return KRON_ERR_NOT_SUPPORTED;
+    SpanCall call;
+    call.D = D;
+    call.es = es;
+    call.N = d.N;
+    call.nx = useful;
+    call.ny = (int64_t)d.ye[0] * d.ye[1] * d.ye[2];
+    call.batch = d.batch;
+    call.square = square;
+    call.up_one = d.ye[0] == d.xe[0] + 1 && d.ye[1] == d.xe[1] + 1 && (D == 2 || d.ye[2] == d.xe[2] + 1);
+    call.beta = d.beta != 0.0;
+    call.x_packed = d.contiguous;
+    call.y_packed = d.ldy == d.ye[0] && (D == 2 || d.ldy2 == d.ye[0] * d.ye[1]) && (d.batch == 1 || d.ldyp == call.ny);
+    call.y_aligned = d.ycontig;
+    call.yvec = d.yvec / es;
+    call.row_bytes = (int)std::min<int64_t>(INT32_MAX, (int64_t)d.ldy * es);
+    if (scalar_body_faster(call)) return KRON_ERR_NOT_SUPPORTED;
     // Offsets of a tile (at most 256 instances) in Y are kept in 32 bits.
     if (d.ldyp >= (int64_t)INT32_MAX / 256) return KRON_ERR_NOT_SUPPORTED;
     SpanArgs a;
@@ -668,8 +675,7 @@ kron_status launch_span(const KronDesc& d, cudaStream_t st) {
     // Instances per tile: about two fibers per thread in the stage with the fewest.
     // (A tuned tile belongs to the contiguous bodies and is not used here.)
     int P = std::max(1, 2 * kSpanThreads / (int)std::min(a.fib[0].d, std::min(a.fib[1].d, D == 3 ? a.fib[2].d : 256u)));
-    const bool packed = d.beta == 0.0 && d.ldy == y1 && (D == 2 || d.ldy2 == y1 * y2) &&
-                        (d.batch == 1 || d.ldyp == a.ny);
+    const bool packed = d.beta == 0.0 && call.y_packed;
     // Chunks of a row of Y: up to 16 bytes, every row of every instance aligned to it.
     a.vec = 1;
     for (int v = 4; v >= 2; v /= 2) {
