@@ -239,14 +239,21 @@ static void choose_yvec(KronDesc& d) {
 // n = 13: 343 -> 221, n = 14: 231 -> 229, n = 15: 223 -> 254 (stays).  16-bit storage 2-D n = 8:
 // 205 -> 143, n = 9: 293 -> 165, n = 10: 127 -> 154 (stays), n = 11: 217 -> 165, n = 13: 162 -> 188
 // (stays); 3-D n = 4: 1683 -> 153, n = 11: 330 -> 246, n = 12: 254 -> 231, n = 13: 256 -> 290 (stays).
-// Only calls that the split path itself takes are served (contiguous operands); with beta != 0
-// the FP32 bodies of 16-bit odd n are slower (old values of Y element by element), so the line
-// lies lower there.
+// Only calls that the split path itself takes are served: packed operands and packed
+// results, the latter at any element alignment, so that the arithmetic of a call does not
+// hang on it except near the line, which lies lower for results off a 16-byte boundary
+// (67 M elements: FP32 2-D n = 14 182 -> 108 us, n = 15 107 -> 117 (stays), 3-D n = 4 1056 -> 137,
+// n = 11 256 -> 149, n = 12 182 -> 201 (stays); 16-bit 3-D n = 11 189 -> 155, n = 12 159 -> 202
+// (stays)).  With beta != 0 odd n of 16-bit storage leaves the split path at n <= 7 only (there
+// 1.6-10 times faster; above, 2-D n = 9 323 -> 179 and 3-D n = 15 434 -> 297 say that the line
+// could lie higher).
 static bool cuda_cores_beat_split(const KronDesc& d) {
-    if (!d.contiguous || !d.ycontig) return false;
+    const int64_t nx = d.D == 2 ? d.N * d.N : d.N * d.N * d.N;
+    const bool y_packed = d.ldy == d.N && (d.D == 2 || d.ldy2 == d.N * d.N) && d.ldyp == nx;
+    if (!d.contiguous || !y_packed) return false;
     if (d.io != KRON_R32F && d.beta != 0.0 && (d.N & 1)) return d.N <= 7;
-    if (d.io == KRON_R32F) return d.D == 2 ? d.N <= 15 : d.N <= 14;
-    return d.D == 2 ? d.N <= 9 || d.N == 11 : d.N <= 12;
+    if (d.io == KRON_R32F) return d.ycontig ? (d.D == 2 ? d.N <= 15 : d.N <= 14) : (d.D == 2 ? d.N <= 14 : d.N <= 11);
+    return d.D == 2 ? d.N <= 9 || d.N == 11 : d.N <= (d.ycontig ? 12 : 11);
 }
 
 static kron_status dispatch(KronDesc& d, cudaStream_t st) {
