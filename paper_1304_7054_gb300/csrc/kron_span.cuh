@@ -77,7 +77,8 @@ struct SpanArgs {
     f2 m[3][8 * kMaxN];           // stage s: rows (2r, 2r+1) of column l at r + 8 l, zero-padded
     const void* X;
     void* Y;
-    int64_t batch, ldxp, ldyp;    // elements
+    int64_t ldxp, ldyp;           // elements
+    int ntiles, last;             // tiles; instances of the last one
     int xs_col, xs_plane;         // strides of the contracted / plane index of X (elements)
     int xspan;                    // elements spanned by one operand
     int head, tail;               // first / last tiles whose copies would reach outside X
@@ -357,10 +358,10 @@ __device__ __forceinline__ void span_copy_out(const SpanArgs& a, int64_t inst0, 
 // Bulk copy of the 16-byte granules that hold tile `tile`'s operand span; the first
 // element sits at the span's own phase in the buffer.
 template <typename S>
-__device__ __forceinline__ void span_issue(const SpanArgs& a, unsigned char* dst, uint64_t* bar, int64_t tile,
+__device__ __forceinline__ void span_issue(const SpanArgs& a, unsigned char* dst, uint64_t* bar, int tile,
                                            uint64_t pol) {
-    const int64_t inst0 = tile * a.P;
-    const int cnt = (int)min((int64_t)a.P, a.batch - inst0);
+    const int64_t inst0 = (int64_t)tile * a.P;
+    const int cnt = tile == a.ntiles - 1 ? a.last : a.P;
     const uintptr_t b0 = (uintptr_t)(static_cast<const S*>(a.X) + inst0 * a.ldxp);
     const uintptr_t b1 = b0 + ((cnt - 1) * a.ldxp + a.xspan) * sizeof(S);
     const uintptr_t a0 = b0 & ~(uintptr_t)15;
@@ -372,10 +373,10 @@ __device__ __forceinline__ void span_issue(const SpanArgs& a, unsigned char* dst
 // As span_issue, for the whole CTA: the copy takes the granules that lie inside the span,
 // the threads load the elements before and after them.  The caller's barrier follows.
 template <typename S>
-__device__ __forceinline__ void span_issue_inside(const SpanArgs& a, unsigned char* dst, uint64_t* bar, int64_t tile,
+__device__ __forceinline__ void span_issue_inside(const SpanArgs& a, unsigned char* dst, uint64_t* bar, int tile,
                                                   uint64_t pol) {
-    const int64_t inst0 = tile * a.P;
-    const int cnt = (int)min((int64_t)a.P, a.batch - inst0);
+    const int64_t inst0 = (int64_t)tile * a.P;
+    const int cnt = tile == a.ntiles - 1 ? a.last : a.P;
     const uintptr_t b0 = (uintptr_t)(static_cast<const S*>(a.X) + inst0 * a.ldxp);
     const uintptr_t b1 = b0 + ((cnt - 1) * a.ldxp + a.xspan) * sizeof(S);
     const uintptr_t from = (b0 + 15) & ~(uintptr_t)15, to = b1 & ~(uintptr_t)15;
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
     // outside, one each; the others walk the tiles between them.
     const int walkers = (int)gridDim.x - a.head - a.tail;
     const int grid = walkers > 0 ? walkers : 1;   // step of the walk
-    int64_t first = a.head + (int)blockIdx.x, end = (a.batch + a.P - 1) / a.P - a.tail;
+    int first = a.head + (int)blockIdx.x, end = a.ntiles - a.tail;
     const bool edge = (int)blockIdx.x >= walkers;
     if (edge) {
         first = (int)blockIdx.x - walkers;
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
         fence_barrier_init();
         pol = l2_evict_first_policy();
         for (int s = 0; s < kSpanRing; ++s) {
-            const int64_t t = first + s * grid;
+            const int t = first + s * grid;
             if (t < end && !edge) span_issue<S>(a, slots + s * a.slot_bytes, &full[s], t, pol);
         }
     }
@@ -423,10 +424,10 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
     __syncthreads();
 
     int it = 0;
-    for (int64_t tile = first; tile < end; tile += grid, ++it) {
+    for (int tile = first; tile < end; tile += grid, ++it) {
         const int s = it % kSpanRing;
-        const int64_t inst0 = tile * a.P;
-        const int cnt = (int)min((int64_t)a.P, a.batch - inst0);
+        const int64_t inst0 = (int64_t)tile * a.P;
+        const int cnt = tile == a.ntiles - 1 ? a.last : a.P;
         unsigned char* slot = slots + s * a.slot_bytes;
         const S* xt = reinterpret_cast<const S*>(
             slot + ((uintptr_t)(static_cast<const S*>(a.X) + inst0 * a.ldxp) & 15u));
@@ -457,7 +458,7 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {   // let in-flight copies land before the CTA exits
                 for (int j = it; j < it + kSpanRing - (it > 0); ++j)
-                    if (tile + (int64_t)(j - it) * grid < end)
+                    if (tile + (j - it) * grid < end)
                         mbar_wait_bounded(&full[j % kSpanRing], (unsigned)(j / kSpanRing) & 1u, a.err);
                 bulk_wait_all();
             }
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(kSpanThreads, 4) span_kernel(const __grid_cons
         }
         // The previous tile's slot: its results have left, the next operands come in.
         if (tid == 0 && it > 0) {
-            const int64_t next = tile + (kSpanRing - 1) * grid;
+            const int next = tile + (kSpanRing - 1) * grid;
             if (next < end) {
                 const int p = (it - 1) % kSpanRing;
                 bulk_wait_read();
@@ -534,7 +535,7 @@ kron_status launch_span_n(const KronDesc& d, const SpanArgs& a, size_t smem, cud
     const DeviceInfo& dev = device_info();
     auto kern = span_kernel<S, NI, NO, D>;
     if (!ensure_smem_optin((const void*)kern, smem)) return KRON_ERR_CUDA;
-    const int64_t ntiles = (d.batch + a.P - 1) / a.P, edges = a.head + a.tail;
+    const int64_t ntiles = a.ntiles, edges = a.head + a.tail;
     int64_t grid = d.grid;
     if (grid <= 0) {
         int per_sm = 0;
@@ -654,7 +655,6 @@ kron_status launch_span(const KronDesc& d, cudaStream_t st) {
         }
     a.X = d.X;
     a.Y = d.Y;
-    a.batch = d.batch;
     a.ldxp = d.ldxp;
     a.ldyp = d.ldyp;
     a.xs_col = d.ldx;
@@ -711,6 +711,10 @@ kron_status launch_span(const KronDesc& d, cudaStream_t st) {
     while (smem > dev.smem_per_block_optin && P > 1) smem = smem_of(--P);
     if (smem > dev.smem_per_block_optin) return KRON_ERR_NOT_SUPPORTED;
     a.P = P;
+    const int64_t ntiles = (d.batch + P - 1) / P;
+    if (ntiles > (1 << 30)) return KRON_ERR_NOT_SUPPORTED;   // tiles are counted in 32 bits
+    a.ntiles = (int)ntiles;
+    a.last = (int)(d.batch - (ntiles - 1) * P);
     const SpanEdges ed = span_edges((uintptr_t)d.X, d.batch, P, d.batch > 1 ? d.ldxp : 0, xspan, es);
     if (!ed.copies) return KRON_ERR_NOT_SUPPORTED;
     a.head = ed.head;
