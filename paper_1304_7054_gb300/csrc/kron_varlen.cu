@@ -41,6 +41,7 @@
 #include "kron_fiber.cuh"
 #include "kron_internal.h"
 #include "kron_pair.cuh"
+#include "kron_varlen_rule.h"
 
 namespace kron {
 
@@ -84,6 +85,7 @@ struct __align__(8) VarlenArgs {
     const void* X;
     void* Y;
     int ntiles;
+    int steal;                // one CTA per tile, running CTAs take over the rest (else the grid walks)
     int alpha_one, beta_zero;  // Y = alpha (K x) + beta Y (beta = 0: Y is not read)
     float alpha, beta;
     unsigned* err;
@@ -396,9 +398,9 @@ __global__ void __launch_bounds__(kVlThreads, 4) varlen_kernel(const __grid_cons
     const int tid = threadIdx.x;
     const int4 none = make_int4(0, 0, 0, 0);
     if ((int)blockIdx.x >= a.ntiles) return;
-    // Thread 0 asks for tiles: one request at a time, none after the first refusal.  A grid
-    // smaller than the list walks it in fixed steps instead.
-    const bool steal = (int)gridDim.x == a.ntiles;
+    // Stealing: thread 0 asks for tiles, one request at a time, none after the first refusal.
+    // Otherwise the grid walks the list in fixed steps.
+    const bool steal = a.steal;
     unsigned clc_phase = 0;
     bool more = true;
     int walk = blockIdx.x;
@@ -581,22 +583,19 @@ static void* vl_kernel_ptr(kron_dtype io) {
     }
 }
 
-// CTAs of the launch.  Code of many large classes (a class's is about 24 bytes times
-// kind n^2) wants the tiles taken in order: one CTA per tile, running CTAs take over the
-// rest.  Below about 17 KB the instruction cache holds all of it, and short tiles are
-// 3-5% faster walked in fixed steps by the resident CTAs (3-D n = 16 alone: 90 us walked,
-// 86 taken in order; n = 6 alone: 68 and 70).
-static int vl_grid(const kron_varlen_plan* p, const void* fn, const DeviceInfo& dev) {
+// CTAs of the launch, and whether they take tiles over (kron_varlen_rule.h).
+static int vl_grid(const kron_varlen_plan* p, const void* fn, const DeviceInfo& dev, int* steal) {
     int units = 0;
     for (int key = 0; key < kVlKeys; ++key) {
         const int n = (key & 15) + 1;
         if (p->present[key]) units += (key < 16 ? 2 : 3) * n * n;
     }
     const int tiles = (int)p->tiles.size();
-    if (units >= 700) return tiles;
     int per_sm = 0;
     if (!resident_ctas(&per_sm, (const void*)fn, kVlThreads, p->smem)) return 0;
-    return std::min(std::max(1, per_sm) * dev.sms, tiles);
+    const int resident = std::max(1, per_sm) * dev.sms;
+    *steal = tiles_taken_over(units, tiles, resident);
+    return *steal ? tiles : std::min(resident, tiles);
 }
 
 // Sort by class, cut tiles, order them largest work first, size the workspace and smem.
@@ -698,7 +697,7 @@ static kron_status vl_launch(kron_varlen_plan* p, const void* X, void* Y, void* 
     }
     kron_status r = vl_fill_args(p, X, Y, ws);
     if (r != KRON_OK) return r;
-    const int grid = vl_grid(p, fn, dev);
+    const int grid = vl_grid(p, fn, dev, &p->args->steal);
     if (grid < 1) return KRON_ERR_CUDA;
     int xbe = p->xbuf_bytes;
     void* kargs[2] = {p->args, &xbe};
@@ -989,7 +988,7 @@ KRON_API kron_status kron_varlen_execute_noalloc(kron_varlen_plan* plan, const v
     if (r != KRON_OK) return r;
     void* fn = vl_kernel_ptr(plan->io);
     if (!ensure_smem_optin(fn, plan->smem)) return KRON_ERR_CUDA;   // the attribute only ever grows
-    const int grid = vl_grid(plan, fn, dev);
+    const int grid = vl_grid(plan, fn, dev, &plan->args->steal);
     if (grid < 1) return KRON_ERR_CUDA;
     int xbe = plan->xbuf_bytes;
     void* kargs[2] = {plan->args, &xbe};
