@@ -85,7 +85,6 @@ struct __align__(8) VarlenArgs {
     const void* X;
     void* Y;
     int ntiles;
-    int steal;                // one CTA per tile, running CTAs take over the rest (else the grid walks)
     int alpha_one, beta_zero;  // Y = alpha (K x) + beta Y (beta = 0: Y is not read)
     float alpha, beta;
     unsigned* err;
@@ -383,7 +382,7 @@ __device__ __forceinline__ int clc_answer(const uint4* res) {
 // of the list, class by class: CTAs that walked fixed shares of it drifted apart until
 // every class's code ran at once and missed the instruction cache (the default workload:
 // 494 us; taken in order 379).
-template <typename S>
+template <typename S, bool STEAL>
 __global__ void __launch_bounds__(kVlThreads, 4) varlen_kernel(const __grid_constant__ VarlenArgs a, int xbuf_bytes) {
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);   // one barrier per operand buffer
@@ -398,19 +397,20 @@ __global__ void __launch_bounds__(kVlThreads, 4) varlen_kernel(const __grid_cons
     const int tid = threadIdx.x;
     const int4 none = make_int4(0, 0, 0, 0);
     if ((int)blockIdx.x >= a.ntiles) return;
-    // Stealing: thread 0 asks for tiles, one request at a time, none after the first refusal.
-    // Otherwise the grid walks the list in fixed steps.
-    const bool steal = a.steal;
+    // STEAL: thread 0 asks for tiles, one request at a time, none after the first refusal.
+    // Otherwise the grid walks the list in fixed steps (a kernel of its own: with the choice
+    // made at run time every walked tile carried the other's code, 2-D n = 6, 100,000
+    // instances 23.1 -> 24.9 us, n = 2..10 27.1 -> 29.0).
     unsigned clc_phase = 0;
     bool more = true;
     int walk = blockIdx.x;
     auto ask = [&]() {
-        if (steal && more) clc_request(clc_res, clc_bar);
+        if (STEAL && more) clc_request(clc_res, clc_bar);
     };
     auto take = [&]() -> int {   // the answer to the request in flight: a tile, or -1
         if (!more) return -1;
         int t = -1;
-        if (steal) {
+        if constexpr (STEAL) {
             if (mbar_wait_bounded(clc_bar, clc_phase, a.err)) t = clc_answer(clc_res);
             clc_phase ^= 1u;
         } else if ((walk += gridDim.x) < a.ntiles) {
@@ -574,28 +574,31 @@ struct kron_varlen_plan {
 
 namespace kron {
 
+template <bool STEAL>
 static void* vl_kernel_ptr(kron_dtype io) {
     switch (io) {
-        case KRON_R32F: return (void*)varlen_kernel<float>;
-        case KRON_R16BF: return (void*)varlen_kernel<__nv_bfloat16>;
-        case KRON_R16F: return (void*)varlen_kernel<__half>;
+        case KRON_R32F: return (void*)varlen_kernel<float, STEAL>;
+        case KRON_R16BF: return (void*)varlen_kernel<__nv_bfloat16, STEAL>;
+        case KRON_R16F: return (void*)varlen_kernel<__half, STEAL>;
         default: return nullptr;
     }
 }
 
-// CTAs of the launch, and whether they take tiles over (kron_varlen_rule.h).
-static int vl_grid(const kron_varlen_plan* p, const void* fn, const DeviceInfo& dev, int* steal) {
+// The kernel of a launch, ready for its shared memory, and its CTAs (0: a CUDA error).
+static int vl_grid(const kron_varlen_plan* p, const DeviceInfo& dev, void** fn) {
     int units = 0;
     for (int key = 0; key < kVlKeys; ++key) {
         const int n = (key & 15) + 1;
         if (p->present[key]) units += (key < 16 ? 2 : 3) * n * n;
     }
     const int tiles = (int)p->tiles.size();
+    *fn = vl_kernel_ptr<false>(p->io);
     int per_sm = 0;
-    if (!resident_ctas(&per_sm, (const void*)fn, kVlThreads, p->smem)) return 0;
+    if (!ensure_smem_optin(*fn, p->smem) || !resident_ctas(&per_sm, *fn, kVlThreads, p->smem)) return 0;
     const int resident = std::max(1, per_sm) * dev.sms;
-    *steal = tiles_taken_over(units, tiles, resident);
-    return *steal ? tiles : std::min(resident, tiles);
+    if (!tiles_taken_over(units, tiles, resident)) return std::min(resident, tiles);
+    *fn = vl_kernel_ptr<true>(p->io);
+    return ensure_smem_optin(*fn, p->smem) ? tiles : 0;
 }
 
 // Sort by class, cut tiles, order them largest work first, size the workspace and smem.
@@ -689,15 +692,14 @@ static kron_status vl_launch(kron_varlen_plan* p, const void* X, void* Y, void* 
     const DeviceInfo& dev = device_info();
     if (dev.sms <= 0) return KRON_ERR_CUDA;
     if (p->smem > dev.smem_per_block_optin) return KRON_ERR_NOT_SUPPORTED;
-    void* fn = vl_kernel_ptr(p->io);
-    if (!ensure_smem_optin(fn, p->smem)) return KRON_ERR_CUDA;
     if (p->uploaded_ws != ws || p->uploaded_version != p->version) {
         kron_status r = vl_upload(p, ws, st);
         if (r != KRON_OK) return r;
     }
     kron_status r = vl_fill_args(p, X, Y, ws);
     if (r != KRON_OK) return r;
-    const int grid = vl_grid(p, fn, dev, &p->args->steal);
+    void* fn = nullptr;
+    const int grid = vl_grid(p, dev, &fn);
     if (grid < 1) return KRON_ERR_CUDA;
     int xbe = p->xbuf_bytes;
     void* kargs[2] = {p->args, &xbe};
@@ -986,9 +988,8 @@ KRON_API kron_status kron_varlen_execute_noalloc(kron_varlen_plan* plan, const v
     if (r != KRON_OK) return r;
     r = vl_fill_args(plan, X, Y, ws);
     if (r != KRON_OK) return r;
-    void* fn = vl_kernel_ptr(plan->io);
-    if (!ensure_smem_optin(fn, plan->smem)) return KRON_ERR_CUDA;   // the attribute only ever grows
-    const int grid = vl_grid(plan, fn, dev, &plan->args->steal);
+    void* fn = nullptr;
+    const int grid = vl_grid(plan, dev, &fn);
     if (grid < 1) return KRON_ERR_CUDA;
     int xbe = plan->xbuf_bytes;
     void* kargs[2] = {plan->args, &xbe};
