@@ -419,8 +419,13 @@ size_t pair_smem_bytes(int P, int nstage) {
 // elements with the second buffer; 3-D n = 8: 80 -> 75, n = 16: 127 -> 117; n = 14: 148 -> 158,
 // so not there); in 2-D a tile is half the bytes of an FP32 one, and twice the instances
 // pay up to n = 10 (n = 4: 78 -> 64 us with a second buffer, n = 6: 67 -> 62, n = 10:
-// 80 -> 67; n = 12: 70 -> 74; at n = 8 the second fiber already does it).  Only with
-// beta = 0: old values of Y read by more fibers at once cost more (n = 4: 86 -> 124 us).
+// 80 -> 67; n = 12: 70 -> 74; at n = 8 the second fiber already does it).  In 2-D only with
+// beta = 0: old values of Y read by more fibers at once cost more (n = 4: 86 -> 124 us); in
+// 3-D, where the tile is the same, with beta != 0 too (33 M elements: n = 4 74.2 -> 73.4, n = 8
+// 68.8 -> 67.7, n = 14, one fiber instead of two, 118 -> 113, n = 16 77.9 -> 78.3).  Up to
+// n = 10 the FP32 choices stay where these would make fewer than two tiles per SM (2-D n = 6,
+// 10,000 instances: 2.7 us with them, 2.4 without; n = 8, one instance: 2.5 and 2.2; 3-D n = 8:
+// 2.8 and 2.6).
 template <int N, int D, int SB>
 struct PairConfig {
     static constexpr int NT = 128;
@@ -465,7 +470,8 @@ kron_status launch_pair_n(const KronDesc& d, cudaStream_t st) {
     a.err = device_error_word();
     if (!a.err) return KRON_ERR_CUDA;
     using Cfg = PairConfig<N, D, (int)sizeof(S)>;
-    const bool plain = sizeof(S) == 2 && D == 2 && d.beta != 0.0;   // the FP32 choices instead
+    const bool few = N <= 10 && d.P <= 0 && (d.batch + Cfg::P0 - 1) / Cfg::P0 < 2 * dev.sms;
+    const bool plain = sizeof(S) == 2 && ((D == 2 && d.beta != 0.0) || few);   // the FP32 choices instead
     int P = d.P > 0 ? d.P : (plain ? PairConfig<N, D, 4>::P0 : Cfg::P0);
     if (!L::XPAD) {
         int mult = 1;
@@ -479,7 +485,7 @@ kron_status launch_pair_n(const KronDesc& d, cudaStream_t st) {
     if (smem > dev.smem_per_block_optin) return KRON_ERR_NOT_SUPPORTED;
     a.P = P;
     a.nstage = nstage;
-    const int fps = d.fps > 0 ? d.fps : (plain ? 1 : Cfg::FPS);
+    const int fps = d.fps > 0 ? d.fps : (plain ? PairConfig<N, D, 4>::FPS : Cfg::FPS);
     auto kern = fps == 2 ? pair_kernel<S, N, D, NT, 2> : pair_kernel<S, N, D, NT, 1>;
     if (!ensure_smem_optin((const void*)kern, smem)) return KRON_ERR_CUDA;
     const int64_t ntiles = (d.batch + P - 1) / P;
