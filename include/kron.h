@@ -365,7 +365,7 @@ KRON_API kron_status kron_autotune(kron_stream_t stream, int kind, int n, int64_
  * values out of range; all-zero restores the built-in default.  Strided,
  * transposed, rectangular or misaligned batches (FP32 or 16-bit storage), and odd n
  * with 16-bit storage, run the general-layout body, or the scalar body where that is
- * set or measured faster.  The 2-D split
+ * set or measured faster (for packed calls of odd n a tile or depth sets it too).  The 2-D split
  * tensor path (KRON_COMPUTE_32F_BF16X3, FP32 or 16-bit storage) has two bodies:
  * KRON_VARIANT_IN_PLACE, one zero-padded 16 x 16 tile per instance (n <= 8:
  * several instances on the tile's diagonal), the second product taking the

@@ -11,6 +11,7 @@
 
 #include "kron_device.cuh"
 #include "kron_internal.h"
+#include "kron_span_rule.h"
 
 namespace kron {
 
@@ -306,7 +307,9 @@ static kron_status dispatch(KronDesc& d, cudaStream_t st) {
         if (r != KRON_ERR_NOT_SUPPORTED) return r;
     }
     // General layouts, and odd n with 16-bit storage.
-    if (d.variant != KRON_VARIANT_SCALAR && (!d.ycontig || ((d.N & 1) && d.io != KRON_R32F && d.beta == 0.0))) {
+    if (d.variant != KRON_VARIANT_SCALAR &&
+        span_body_asked(d.ycontig, d.N, d.io == KRON_R16BF || d.io == KRON_R16F, d.beta != 0.0,
+                        d.P > 0 || d.nstage >= 0)) {
         kron_status r = KRON_ERR_NOT_SUPPORTED;
         switch (d.io) {
             case KRON_R32F: r = d.D == 2 ? launch_span_f32_d2(d, st) : launch_span_f32_d3(d, st); break;

@@ -68,4 +68,11 @@ inline bool scalar_body_faster(const SpanCall& c) {
     return c.x_packed && c.D == 3 && c.N == 12 && c.yvec >= 2;
 }
 
+// Whether the span body is asked at all: every general layout, and packed calls of odd n
+// with 16-bit storage and beta = 0, unless a tile or a depth is set for them (those are the
+// scalar body's).
+inline bool span_body_asked(bool y_aligned, int N, bool half, bool beta, bool tile_set) {
+    return !y_aligned || (N % 2 == 1 && half && !beta && !tile_set);
+}
+
 }  // namespace kron
