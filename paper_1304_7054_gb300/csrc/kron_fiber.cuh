@@ -530,9 +530,15 @@ kron_status launch_fiber_n(const KronDesc& d, cudaStream_t st) {
         }
     };
     for (int e = 0; e < N * N; ++e) {
-        a.m1[e] = elem(d.m1[e], d.m1i[e]);
-        a.m2[e] = elem(d.m2[e], d.m2i[e]);
-        if constexpr (D == 3) a.m3[e] = elem(d.m3[e], d.m3i[e]);
+        if constexpr (is_cplx<T>::value) {
+            a.m1[e] = elem(d.m1[e], d.m1i[e]);
+            a.m2[e] = elem(d.m2[e], d.m2i[e]);
+            if constexpr (D == 3) a.m3[e] = elem(d.m3[e], d.m3i[e]);
+        } else {   // (the imaginary parts are not set for real storage)
+            a.m1[e] = elem(d.m1[e], 0.0);
+            a.m2[e] = elem(d.m2[e], 0.0);
+            if constexpr (D == 3) a.m3[e] = elem(d.m3[e], 0.0);
+        }
     }
     if constexpr (D == 2) a.m3[0] = T(0);
     a.X = d.X;
