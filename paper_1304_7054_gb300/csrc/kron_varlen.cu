@@ -71,14 +71,8 @@ __host__ __device__ constexpr int vl_kp(int n) {
     return vl_rows(n) + ((vl_rows(n) % 4 == 2) ? 0 : 2);
 }
 
-struct VlClass {
-    int P;              // instances per tile (0 = class absent)
-    unsigned inv;       // ceil(2^32 / n^kind): exact quotient e / n^kind for e < 4096
-};
-
 struct __align__(8) VarlenArgs {
     float coef[kVlCoef];      // 8-byte aligned: read as coefficient pairs
-    VlClass cls[kVlKeys];
     const int4* tiles;
     const int64_t* xoff;
     const int64_t* yoff;
@@ -640,12 +634,6 @@ static kron_status vl_build(kron_varlen_plan* p) {
 
 static kron_status vl_fill_args(kron_varlen_plan* p, const void* X, void* Y, void* ws) {
     VarlenArgs& a = *p->args;
-    for (int key = 0; key < kVlKeys; ++key) {
-        const int kind = key < 16 ? 2 : 3, n = (key & 15) + 1;
-        const unsigned nx = kind == 2 ? n * n : n * n * n;
-        a.cls[key].P = p->present[key] ? p->P[key] : 0;
-        a.cls[key].inv = nx == 1 ? 0u : (unsigned)((0x100000000ull + nx - 1) / nx);
-    }
     char* w = static_cast<char*>(ws);
     a.tiles = reinterpret_cast<const int4*>(w);
     a.xoff = reinterpret_cast<const int64_t*>(w + round_up(p->order.size() * sizeof(int4), 256));
