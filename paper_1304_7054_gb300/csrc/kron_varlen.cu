@@ -526,7 +526,8 @@ static int vl_max_P(int kind, int n, size_t es, int xbudget, int ebudget) {
 // many as two rounds of fibers (one per thread) cover in 3-D (a second round halves the
 // share of the barrier waits).  In 2-D one round, or two where the class then still has
 // two tiles for each of four CTAs on 152 SMs (n = 6, 833,333 instances: 163 -> 135 us;
-// in the mixed batch of 200,000 two rounds measured 1% slower).
+// in the mixed batch of 200,000 two rounds measured 1% slower).  The SM count is that of the
+// GPU this is written for: creating a plan touches no device.
 static int vl_default_P(int kind, int n, size_t es, int64_t count) {
     auto fit = [&](int fibers) { return std::max(1, std::min(fibers, vl_max_P(kind, n, es, kVlXBytes, kVlEBytes))); };
     const int two = fit(2 * kVlThreads / (kind == 2 ? n : n * n));
