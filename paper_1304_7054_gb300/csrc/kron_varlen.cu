@@ -394,17 +394,21 @@ __global__ void __launch_bounds__(kVlThreads, 4) varlen_kernel(const __grid_cons
     // STEAL: thread 0 asks for tiles, one request at a time, none after the first refusal.
     // Otherwise the grid walks the list in fixed steps (a kernel of its own: with the choice
     // made at run time every walked tile carried the other's code, 2-D n = 6, 100,000
-    // instances 23.1 -> 24.9 us, n = 2..10 27.1 -> 29.0).
+    // instances 23.1 -> 24.9 us, n = 2..10 27.1 -> 29.0).  For FP32 the stealing kernel
+    // compares the grid with the list again, which always holds: left to fold the walk away,
+    // the compiler gives a slower body (200,000 instances: 377.4 and 379.6 us; bf16 396.3
+    // and 387.4).
+    const bool steal = STEAL && (sizeof(S) == 2 || (int)gridDim.x == a.ntiles);
     unsigned clc_phase = 0;
     bool more = true;
     int walk = blockIdx.x;
     auto ask = [&]() {
-        if (STEAL && more) clc_request(clc_res, clc_bar);
+        if (steal && more) clc_request(clc_res, clc_bar);
     };
     auto take = [&]() -> int {   // the answer to the request in flight: a tile, or -1
         if (!more) return -1;
         int t = -1;
-        if constexpr (STEAL) {
+        if (steal) {
             if (mbar_wait_bounded(clc_bar, clc_phase, a.err)) t = clc_answer(clc_res);
             clc_phase ^= 1u;
         } else if ((walk += gridDim.x) < a.ntiles) {
