@@ -46,13 +46,16 @@ inline bool scalar_body_faster(const SpanCall& c) {
     }
     // Operands that the scalar body copies in bulk too: what is left is how Y is written.
     if (c.x_packed && c.beta) {
-        // old values: misaligned or padded Y, large FP32 2-D n = 5: 1.5, 9: 1.2-1.3, 12: 0.7-0.9,
-        // 13: 1.0-1.1; 3-D n = 7: 1.3-1.7, 12: 1.0-1.7, 14: 1.25, 16: 0.8-1.0; 16-bit 2-D n = 5-8:
-        // 0.95-1.4, 12: 0.6-0.9; 3-D n = 5: 1.3-1.4, 13: 1.1-1.3, 16: 0.5-1.0.  100 instances: all
-        // n 1.0-1.5.
-        if (c.D == 3) return c.N <= 14 || E < (1 << 19);
-        if (c.es == 4) return (c.N >= 3 && c.N <= 11) || c.N == 13 || E < (1 << 17);
-        return (c.N >= 5 && c.N <= 8) || E < (1 << 19);
+        // Old values, large: FP32 2-D n = 5: 1.5, 9: 1.2-1.3, 11: packed Y 1.03, padded 0.86-0.98,
+        // 12: 0.7-0.9, 13: 1.0-1.1; 3-D n = 7: 1.3-1.7, 12: 1.0-1.7, 14: 1.25, 15: packed 1.07-1.16,
+        // padded 0.9, 16: 0.8-1.0; 16-bit 2-D n = 5-8: 0.95-1.4, 9: packed 1.06-1.24, padded
+        // 0.7-0.9, 12: 0.6-1.04, 10, 14, 16 with vector stores 1.07-1.28, without 0.5-0.95; 3-D
+        // n = 5: 1.3-1.4, 13: 1.1-1.3, 16: 0.5-1.0.  100 instances: all n 1.0-1.5.
+        if (c.D == 3) return c.N <= (c.y_packed ? 15 : 14) || E < (1 << 19);
+        if (c.es == 4)
+            return (c.N >= 3 && c.N <= 9) || (c.y_packed && (c.N <= 11 || c.N == 13) && c.N >= 3) || E < (1 << 17);
+        return (c.N >= 5 && c.N <= 8) || (c.y_packed && c.N == 9) ||
+               (c.yvec >= 2 && (c.N == 10 || c.N >= 14)) || E < (1 << 19);
     }
     if (c.x_packed && !c.y_packed) {
         // Y with gaps.  3-D n = 5: 1.0-1.4, n = 8: 0.75-1.06, n = 9-13 in FP32 1.0-1.15 (11: 0.9-1.0),

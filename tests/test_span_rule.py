@@ -42,12 +42,15 @@ SCALAR = [(2, 4, 7, 7, None, 1, MISALIGNED), (3, 4, 12, 12, None, 1, MISALIGNED)
           (3, 2, 6, 6, None, 0, PADDED), (2, 4, 4, 4, 4, 0, ROWS), (3, 4, 3, 3, 16, 0, ROWS), (2, 2, 2, 2, 2000, 0, ROWS),
           (3, 2, 5, 9, 100, 0, ROWS), (3, 2, 3, 7, 2000, 0, ROWS), (3, 2, 6, 7, None, 1, ROWS), (2, 2, 5, 6, None, 1, ROWS),
           (3, 2, 13, 14, None, 1, ROWS), (3, 4, 6, 6, None, 1, ROWS), (3, 4, 1, 1, None, 0, ROWS),
-          (3, 2, 6, 10, 100, 0, ROWS), (2, 2, 13, 11, 4, 0, ROWS)]
-SPAN = [(2, 4, 16, 16, None, 1, MISALIGNED), (3, 4, 16, 16, None, 1, MISALIGNED), (2, 2, 12, 12, None, 1, PADDED),
+          (3, 2, 6, 10, 100, 0, ROWS), (2, 2, 13, 11, 4, 0, ROWS), (2, 2, 9, 9, None, 1, MISALIGNED),
+          (3, 2, 15, 15, None, 1, MISALIGNED), (2, 2, 14, 14, None, 1, {"x_packed": 1, "y_packed": 1, "yvec": 2})]
+SPAN = [(2, 4, 16, 16, None, 1, MISALIGNED), (2, 2, 9, 9, None, 1, PADDED), (2, 4, 11, 11, None, 1, PADDED),
+        (3, 4, 16, 16, None, 1, MISALIGNED), (2, 2, 12, 12, None, 1, PADDED),
         (2, 4, 7, 7, None, 0, MISALIGNED), (3, 2, 9, 9, None, 0, MISALIGNED), (2, 4, 12, 12, None, 0, PADDED),
         (2, 4, 7, 7, None, 1, ROWS), (3, 4, 8, 8, 100, 0, ROWS), (3, 4, 8, 12, 100, 0, ROWS), (2, 4, 4, 5, 2000, 0, ROWS),
         (3, 2, 12, 10, None, 1, ROWS), (3, 2, 13, 14, None, 0, ROWS), (2, 2, 14, 16, None, 0, ROWS),
-        (2, 2, 14, 15, None, 1, ROWS), (3, 2, 16, 14, None, 0, ROWS),
+        (2, 2, 14, 15, None, 1, ROWS), (2, 2, 14, 14, None, 1, MISALIGNED), (3, 2, 15, 15, None, 1, PADDED),
+        (3, 2, 16, 14, None, 0, ROWS),
         (3, 2, 7, 7, 40, 0, {"x_packed": 1, "y_packed": 1, "y_aligned": 1}),
         (2, 2, 3, 3, 1, 0, {"x_packed": 1, "y_packed": 1, "y_aligned": 1})]
 
